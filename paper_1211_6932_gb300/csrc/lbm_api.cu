@@ -44,6 +44,10 @@ struct Batch {
   std::vector<InstParams> inst;  // storage dimensions (axes exchanged where tr[i])
   std::vector<char> tr;          // instance stored transposed (lbm_instance.layout)
   std::vector<int> active;
+  // Viscosity rule of the pair kernel's steps (PAIR_ANY unless every instance has the same
+  // rule, b, G and rates) and the constants the instances share.
+  int rule = lbm::PAIR_ANY;
+  lbm::PairConsts shared{};
   std::vector<long long> steps;
   std::vector<char> dinf_valid;
   InstParams* d_inst = nullptr;
@@ -431,7 +435,7 @@ bool persist_items_ok(const Batch* b, int rows) {
     if (b->active[i])
       items += (long long)lbm::strips_for(b->inst[i].nx, nt, b->vec) *
                ((b->inst[i].ny + rows - 1) / rows);
-  return items >= 2LL * lbm::persist_occupancy(nt, kind) * std::max(b->sms, 1);
+  return items >= 2LL * lbm::persist_occupancy(b->rule, nt, kind) * std::max(b->sms, 1);
 }
 
 // Rows per CTA sweep: about six waves of resident CTAs (measured best on 4096^2: fewer
@@ -446,7 +450,8 @@ int default_rows(const Batch* b) {
     if (b->active[i]) {
       const int nt = step_nt(b, i);
       const int occ = b->fp64 ? lbm::sweep_occupancy<double>(nt, b->vec)
-                              : lbm::sweep_occupancy<float>(nt, b->vec);
+                      : b->vec == 2 ? lbm::pair_occupancy(b->rule, nt)
+                                    : lbm::sweep_occupancy<float>(nt, b->vec);
       sm_rows += (double)lbm::strips_for(b->inst[i].nx, nt, b->vec) * b->inst[i].ny /
                  std::max(occ, 1);
     }
@@ -604,7 +609,7 @@ int build_persist(Batch* b) {
   b->persist_kind = kind;
   b->persist_sync = sync;
   b->persist_grid =
-      std::max(1, std::min(lbm::persist_occupancy(nt, kind) * std::max(b->sms, 1), n));
+      std::max(1, std::min(lbm::persist_occupancy(b->rule, nt, kind) * std::max(b->sms, 1), n));
   if (2 * n > b->cap_items2 || !b->d_items2) {
     free_dev(b->d_items2);
     free_dev(b->d_links2);
@@ -738,6 +743,17 @@ int fill_params(std::string& err, InstParams& P, const lbm_instance& in, bool fp
   return LBM_OK;
 }
 
+// The pair kernel's rule and shared constants for the instances' parameters.
+void set_rule(Batch* b) {
+  const InstParams& A = b->inst[0];
+  b->rule = A.visc_mode;
+  for (const InstParams& P : b->inst) {
+    bool same = P.visc_mode == A.visc_mode && P.b4 == A.b4 && P.G == A.G;
+    for (int k = 0; k < lbm::Q; ++k) same &= P.s[k] == A.s[k];
+    if (!same) b->rule = lbm::PAIR_ANY;
+  }
+  b->shared = lbm::pair_params(A);
+}
 
 int create_batch(Batch* b, int n, const lbm_instance* in, bool fp64, int psi_fp64,
                  void* stream, int device, int nt, int vec, int rows) {
@@ -778,6 +794,7 @@ int create_batch(Batch* b, int n, const lbm_instance* in, bool fp64, int psi_fp6
   }
   b->slab_elems = off;
   b->dense_elems = dense;
+  set_rule(b);
   b->nt = nt_;
   b->vec = vec_;
   b->rows_req = rows;
@@ -829,6 +846,9 @@ int launch_group(Batch* b, int g, int c, cudaStream_t st) {
     e = lbm::launch_sweep<double>(b->grp_nt[g], b->vec, lbm::MODE_STEP, 0,
                                   (const double*)b->slab[c], (double*)b->slab[c ^ 1], b->d_inst,
                                   items, n, mo, b->d_status, st);
+  } else if (b->vec == 2) {
+    e = lbm::launch_pair(b->rule, b->grp_nt[g], b->grp_full[g], (const float*)b->slab[c],
+                         (float*)b->slab[c ^ 1], b->d_inst, items, n, b->d_status, b->shared, st);
   } else {
     MomArgs<float> mo{};
     e = lbm::launch_sweep<float>(b->grp_nt[g], b->vec, lbm::MODE_STEP, b->grp_full[g],
@@ -845,10 +865,10 @@ int launch_group(Batch* b, int g, int c, cudaStream_t st) {
 int launch_persist_steps(Batch* b, int c, int n, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(b->d_sync, 0, sizeof(int) * b->persist_sync, st);
   if (e == cudaSuccess)
-    e = lbm::launch_persist(b->grp_nt[0], b->persist_kind, (float*)b->slab[c],
+    e = lbm::launch_persist(b->rule, b->grp_nt[0], b->persist_kind, (float*)b->slab[c],
                             (float*)b->slab[c ^ 1], b->d_inst, b->d_items2, b->d_links2,
                             b->n_items, n, b->d_sync, b->d_sync + 1, b->d_status,
-                            b->persist_grid, lbm::DEP_WAIT_LIMIT, st);
+                            b->persist_grid, lbm::DEP_WAIT_LIMIT, b->shared, st);
   if (e != cudaSuccess)
     return set_err(b->err, LBM_ECUDA, "persistent step launch failed: %s", cudaGetErrorString(e));
   return LBM_OK;
@@ -2030,11 +2050,11 @@ int lbm_selftest_dep_timeout(lbm_handle* h, int polls) {
     e = cudaMemcpyAsync(d_links2, links2, sizeof(links2), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(sync, 0, 4 * sizeof(int), b->stream);
   if (e == cudaSuccess)
-    e = lbm::launch_persist(b->grp_nt[0],
+    e = lbm::launch_persist(b->rule, b->grp_nt[0],
                             b->grp_full[0] ? lbm::PERSIST_FULL : lbm::PERSIST_STRIP,
                             (float*)b->slab[b->cur], (float*)b->slab[b->cur ^ 1], b->d_inst,
                             d_items2, d_links2, 1, 2,
-                            sync, sync + 1, b->d_status, 1, polls, b->stream);
+                            sync, sync + 1, b->d_status, 1, polls, b->shared, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   dev_free(buf);
   if (e != cudaSuccess)

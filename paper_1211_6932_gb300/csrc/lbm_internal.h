@@ -8,13 +8,35 @@ namespace lbm {
 
 // Launch the fused sweep (MODE_STEP) or the moments/diagnostics pass (MODE_MOMENTS) over
 // n_items work items; nt (threads per CTA), vec (columns per thread) and, for the pair
-// kernel (vec 2), full (full-width strips, see strips_for) select the instantiation.  A
-// pair-kernel CTA whose instance is not of the launched kind returns at once.
+// kernel (vec 2, moments only: its steps are launch_pair), full (full-width strips, see
+// strips_for) select the instantiation.  A pair-kernel CTA whose instance is not of the
+// launched kind returns at once.
 template <typename S>
 cudaError_t launch_sweep(int nt, int vec, int mode, int full, const S* fin, S* fout,
                          const InstParams* d_inst,
                          const WorkItem* d_items, int n_items, const MomArgs<S>& mo,
                          int* d_status, cudaStream_t st);
+// Step of the pair kernel (vec 2) for a viscosity rule (VISC_* with the constants that the
+// instances of the launch share, or PAIR_ANY).
+cudaError_t launch_pair(int rule, int nt, int full, const float* fin, float* fout,
+                        const InstParams* d_inst, const WorkItem* d_items, int n_items,
+                        int* d_status, const PairConsts& shared, cudaStream_t st);
+template <int RULE>
+cudaError_t launch_pair_step(int nt, int full, const float* fin, float* fout,
+                             const InstParams* d_inst, const WorkItem* d_items, int n_items,
+                             int* d_status, const PairConsts& shared, cudaStream_t st);
+template <int RULE>
+cudaError_t launch_pair_persist(int nt, int kind, float* slab0, float* slab1,
+                                const InstParams* d_inst, const WorkItem* items2,
+                                const ItemLink* links2, int n_items, int steps, int* queue,
+                                int* done, int* d_status, int grid, int dep_limit,
+                                const PairConsts& shared, cudaStream_t st);
+template <int RULE>
+int pair_persist_occupancy(int nt, int kind);
+template <int RULE>
+int pair_step_occupancy(int nt);
+// Resident CTAs per SM of the pair kernel's step (at least 1).
+int pair_occupancy(int rule, int nt);
 template <typename S>
 cudaError_t launch_fill_ghosts(S* buf, const InstParams& P, cudaStream_t st);
 template <typename S>
@@ -66,12 +88,13 @@ cudaError_t launch_pressure(const S* rho, const InstParams& P, double sigma, dou
 // item's kind from its instance's width).  items2 and links2 hold 2 n_items entries (the
 // even steps' list, then the odd steps'); queue (one int) and done (one int per chunk)
 // must be zero at launch; dep_limit bounds each dependency wait (DEP_WAIT_LIMIT).
-cudaError_t launch_persist(int nt, int kind, float* slab0, float* slab1,
+cudaError_t launch_persist(int rule, int nt, int kind, float* slab0, float* slab1,
                            const InstParams* d_inst, const WorkItem* items2,
                            const ItemLink* links2, int n_items, int steps, int* queue,
-                           int* done, int* d_status, int grid, int dep_limit, cudaStream_t st);
+                           int* done, int* d_status, int grid, int dep_limit,
+                           const PairConsts& shared, cudaStream_t st);
 // Resident CTAs per SM of the persistent pair kernel of width nt and that kind (at least 1).
-int persist_occupancy(int nt, int kind);
+int persist_occupancy(int rule, int nt, int kind);
 
 // Status bit of an asynchronous initialisation whose fields failed the validity check
 // (host-side status only; distinct from the kernels' STATUS_* bits).

@@ -47,78 +47,6 @@ static cudaError_t launch_sweep_mode(int mode, const S* fin, S* fout, const Inst
                                                d_status, st);
 }
 
-// FP32 pair kernel (two columns per thread, packed float2 arithmetic), strip or
-// full-width instantiation.
-template <int NT, int MODE, bool FULL>
-static cudaError_t launch_sweep2_cfg(const float* fin, float* fout, const InstParams* d_inst,
-                                     const WorkItem* d_items, int n_items,
-                                     const MomArgs<float>& mo, int* d_status, cudaStream_t st) {
-  constexpr size_t smem = Sweep2Cfg<NT>::BYTES;
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = ensure_smem_attr(sweep2_kernel<NT, MODE, FULL>, smem, done);
-  if (e != cudaSuccess) return e;
-  if (n_items <= 0) return cudaSuccess;
-  sweep2_kernel<NT, MODE, FULL><<<n_items, NT, smem, st>>>(fin, fout, d_inst, d_items, n_items,
-                                                           mo, d_status);
-  return cudaGetLastError();
-}
-
-template <int NT>
-static cudaError_t launch_sweep2_mode(int mode, int full, const float* fin, float* fout,
-                                      const InstParams* d_inst, const WorkItem* d_items,
-                                      int n_items, const MomArgs<float>& mo, int* d_status,
-                                      cudaStream_t st) {
-  if (mode == MODE_STEP)
-    return full ? launch_sweep2_cfg<NT, MODE_STEP, true>(fin, fout, d_inst, d_items, n_items,
-                                                         mo, d_status, st)
-                : launch_sweep2_cfg<NT, MODE_STEP, false>(fin, fout, d_inst, d_items, n_items,
-                                                          mo, d_status, st);
-  return full ? launch_sweep2_cfg<NT, MODE_MOMENTS, true>(fin, fout, d_inst, d_items, n_items,
-                                                          mo, d_status, st)
-              : launch_sweep2_cfg<NT, MODE_MOMENTS, false>(fin, fout, d_inst, d_items, n_items,
-                                                           mo, d_status, st);
-}
-
-// Persistent pair kernel (sweep2_persist_kernel) with `grid` CTAs.
-template <int NT, int KIND>
-static cudaError_t launch_persist2_cfg(float* slab0, float* slab1, const InstParams* d_inst,
-                                       const WorkItem* items2, const ItemLink* links2,
-                                       int n_items, int steps, int* queue, int* done,
-                                       int* d_status, int grid, int dep_limit,
-                                       cudaStream_t st) {
-  constexpr size_t smem = Sweep2Cfg<NT>::BYTES;
-  static std::atomic<unsigned long long> flag{0};
-  cudaError_t e = ensure_smem_attr(sweep2_persist_kernel<NT, KIND>, smem, flag);
-  if (e != cudaSuccess) return e;
-  if (n_items <= 0 || steps <= 0 || grid <= 0) return cudaSuccess;
-  sweep2_persist_kernel<NT, KIND><<<grid, NT, smem, st>>>(slab0, slab1, d_inst, items2, links2,
-                                                          n_items, steps, queue, done,
-                                                          d_status, dep_limit);
-  return cudaGetLastError();
-}
-
-template <int NT, int KIND>
-static int persist_occupancy_cfg() {
-  constexpr size_t smem = Sweep2Cfg<NT>::BYTES;
-  cudaFuncSetAttribute(sweep2_persist_kernel<NT, KIND>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int occ = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &occ, sweep2_persist_kernel<NT, KIND>, NT, smem);
-  return (e == cudaSuccess && occ > 0) ? occ : 1;
-}
-
-template <int NT>
-static int occupancy2_cfg() {
-  constexpr size_t smem = Sweep2Cfg<NT>::BYTES;
-  cudaFuncSetAttribute(sweep2_kernel<NT, MODE_STEP, false>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int occ = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &occ, sweep2_kernel<NT, MODE_STEP, false>, NT, smem);
-  return (e == cudaSuccess && occ > 0) ? occ : 1;
-}
-
 template <typename S, int NT>
 static int occupancy_cfg() {
   constexpr size_t smem = SweepCfg<S, NT>::BYTES;
