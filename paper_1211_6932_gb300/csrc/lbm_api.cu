@@ -48,6 +48,10 @@ struct Batch {
   // rule, b, G and rates) and the constants the instances share.
   int rule = lbm::PAIR_ANY;
   lbm::PairConsts shared{};
+  // Tensor maps of the pair kernel's row copies, for the widths of the step launches and of
+  // the moments pass; those of several instances lie in d_maps (2 n_inst each).
+  lbm::RowMaps maps_step{}, maps_mom{};
+  CUtensorMap* d_maps = nullptr;
   std::vector<long long> steps;
   std::vector<char> dinf_valid;
   InstParams* d_inst = nullptr;
@@ -296,6 +300,7 @@ void destroy_batch(Batch* b) {
     if (s) cudaStreamSynchronize(s);
   drop_graphs(b);
   free_dev(b->d_inst);
+  free_dev(b->d_maps);
   free_dev(b->d_items);
   free_dev(b->d_items2);
   free_dev(b->d_links2);
@@ -449,9 +454,9 @@ int default_rows(const Batch* b) {
   for (int i = 0; i < b->n_inst; ++i)
     if (b->active[i]) {
       const int nt = step_nt(b, i);
-      const int occ = b->fp64 ? lbm::sweep_occupancy<double>(nt, b->vec)
+      const int occ = b->fp64 ? lbm::sweep_occupancy<double>(nt)
                       : b->vec == 2 ? lbm::pair_occupancy(b->rule, nt)
-                                    : lbm::sweep_occupancy<float>(nt, b->vec);
+                                    : lbm::sweep_occupancy<float>(nt);
       sm_rows += (double)lbm::strips_for(b->inst[i].nx, nt, b->vec) * b->inst[i].ny /
                  std::max(occ, 1);
     }
@@ -630,6 +635,71 @@ int build_persist(Batch* b) {
   return LBM_OK;
 }
 
+// cuTensorMapEncodeTiled through the runtime's driver entry point (no link against libcuda).
+typedef CUresult (*TensorMapEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
+                                      const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                      const cuuint32_t*, CUtensorMapInterleave,
+                                      CUtensorMapSwizzle, CUtensorMapL2promotion,
+                                      CUtensorMapFloatOOBfill);
+TensorMapEncodeFn tensor_map_encoder() {
+  static std::once_flag once;
+  static TensorMapEncodeFn fn = nullptr;
+  std::call_once(once, [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
+                                         &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = (TensorMapEncodeFn)p;
+  });
+  return fn;
+}
+
+// Tensor map of instance P's rows in a slab for CTAs of nt threads: elements are pairs of
+// floats (a box may have 256 elements a side, a 128-thread row has 260 floats), and rows are
+// copied from a column that is a multiple of four floats, so every copy starts on 16 bytes.
+int row_map(Batch* b, const InstParams& P, float* slab, int nt, CUtensorMap* map) {
+  TensorMapEncodeFn encode = tensor_map_encoder();
+  if (!encode) return set_err(b->err, LBM_ECUDA, "cuTensorMapEncodeTiled is not available");
+  const cuuint64_t dim[3] = {(cuuint64_t)P.pitch / 2, (cuuint64_t)P.ny, (cuuint64_t)lbm::Q};
+  const cuuint64_t stride[2] = {(cuuint64_t)P.pitch * sizeof(float),
+                                (cuuint64_t)P.plane * sizeof(float)};
+  const cuuint32_t box[3] = {(cuuint32_t)(2 * nt + 4) / 2, 1, (cuuint32_t)lbm::Q};
+  const cuuint32_t one[3] = {1, 1, 1};
+  const CUresult r =
+      encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, slab + P.off, dim, stride, box, one,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS)
+    return set_err(b->err, LBM_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
+  return LBM_OK;
+}
+
+// Tensor maps for the current widths (pair tilings only).
+int build_maps(Batch* b) {
+  if (b->fp64 || b->vec != 2) return LBM_OK;
+  const int n = b->n_inst;
+  std::vector<CUtensorMap> maps(4 * (size_t)n);  // step maps (2 i + slab), then moments maps
+  for (int i = 0; i < n; ++i)
+    for (int k = 0; k < 2; ++k) {
+      int rc = row_map(b, b->inst[i], (float*)b->slab[k], step_nt(b, i), &maps[2 * i + k]);
+      if (rc == LBM_OK)
+        rc = row_map(b, b->inst[i], (float*)b->slab[k], mom_nt(b), &maps[2 * (n + i) + k]);
+      if (rc) return rc;
+    }
+  for (int k = 0; k < 2; ++k) {
+    b->maps_step.own[k] = maps[k];
+    b->maps_mom.own[k] = maps[2 * n + k];
+  }
+  if (n == 1) return LBM_OK;
+  if (!b->d_maps) CK(b, dev_malloc(&b->d_maps, sizeof(CUtensorMap) * maps.size()));
+  CK(b, cudaMemcpy(b->d_maps, maps.data(), sizeof(CUtensorMap) * maps.size(),
+                   cudaMemcpyHostToDevice));
+  b->maps_step.table = b->d_maps;
+  b->maps_mom.table = b->d_maps + 2 * n;
+  return LBM_OK;
+}
+
 // Rebuild and upload the work lists (after a tiling change or a retirement).
 int rebuild_items(Batch* b) {
   drop_graphs(b);
@@ -637,6 +707,10 @@ int rebuild_items(Batch* b) {
   if (per_instance(b)) {
     b->inst_nt.resize(b->n_inst);
     for (int i = 0; i < b->n_inst; ++i) b->inst_nt[i] = pair_threads_for(b->inst[i].nx);
+  }
+  {
+    int rc = build_maps(b);
+    if (rc) return rc;
   }
   b->rows = b->rows_req > 0 ? b->rows_req : default_rows(b);
   make_step_items(b);
@@ -843,17 +917,16 @@ int launch_group(Batch* b, int g, int c, cudaStream_t st) {
   cudaError_t e;
   if (b->fp64) {
     MomArgs<double> mo{};
-    e = lbm::launch_sweep<double>(b->grp_nt[g], b->vec, lbm::MODE_STEP, 0,
-                                  (const double*)b->slab[c], (double*)b->slab[c ^ 1], b->d_inst,
-                                  items, n, mo, b->d_status, st);
+    e = lbm::launch_sweep<double>(b->grp_nt[g], lbm::MODE_STEP, (const double*)b->slab[c],
+                                  (double*)b->slab[c ^ 1], b->d_inst, items, n, mo, b->d_status,
+                                  st);
   } else if (b->vec == 2) {
-    e = lbm::launch_pair(b->rule, b->grp_nt[g], b->grp_full[g], (const float*)b->slab[c],
+    e = lbm::launch_pair(b->rule, b->grp_nt[g], b->grp_full[g], b->maps_step, c,
                          (float*)b->slab[c ^ 1], b->d_inst, items, n, b->d_status, b->shared, st);
   } else {
     MomArgs<float> mo{};
-    e = lbm::launch_sweep<float>(b->grp_nt[g], b->vec, lbm::MODE_STEP, b->grp_full[g],
-                                 (const float*)b->slab[c], (float*)b->slab[c ^ 1], b->d_inst,
-                                 items, n, mo, b->d_status, st);
+    e = lbm::launch_sweep<float>(b->grp_nt[g], lbm::MODE_STEP, (const float*)b->slab[c],
+                                 (float*)b->slab[c ^ 1], b->d_inst, items, n, mo, b->d_status, st);
   }
   if (e != cudaSuccess)
     return set_err(b->err, LBM_ECUDA, "step kernel launch failed: %s", cudaGetErrorString(e));
@@ -865,7 +938,8 @@ int launch_group(Batch* b, int g, int c, cudaStream_t st) {
 int launch_persist_steps(Batch* b, int c, int n, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(b->d_sync, 0, sizeof(int) * b->persist_sync, st);
   if (e == cudaSuccess)
-    e = lbm::launch_persist(b->rule, b->grp_nt[0], b->persist_kind, (float*)b->slab[c],
+    e = lbm::launch_persist(b->rule, b->grp_nt[0], b->persist_kind, b->maps_step, c,
+                            (float*)b->slab[c],
                             (float*)b->slab[c ^ 1], b->d_inst, b->d_items2, b->d_links2,
                             b->n_items, n, b->d_sync, b->d_sync + 1, b->d_status,
                             b->persist_grid, lbm::DEP_WAIT_LIMIT, b->shared, st);
@@ -1214,18 +1288,24 @@ int get_pops(Batch* b, int i, double* f) {
 // Launch the moments/diagnostics kernel over a device list of n items on the batch's
 // stream.  The pair kernel has strip and full-width instantiations: both are launched over
 // the whole list, and each CTA works only on an item of its own kind.
-template <typename S>
 cudaError_t launch_moments(const Batch* b, const WorkItem* d_items, int n,
-                           const MomArgs<S>& mo) {
+                           const MomArgs<double>& mo) {
+  return lbm::launch_sweep<double>(mom_nt(b), lbm::MODE_MOMENTS, (const double*)b->slab[b->cur],
+                                   nullptr, b->d_inst, d_items, n, mo, b->d_status, b->stream);
+}
+cudaError_t launch_moments(const Batch* b, const WorkItem* d_items, int n,
+                           const MomArgs<float>& mo) {
+  if (b->vec != 2)
+    return lbm::launch_sweep<float>(mom_nt(b), lbm::MODE_MOMENTS, (const float*)b->slab[b->cur],
+                                    nullptr, b->d_inst, d_items, n, mo, b->d_status, b->stream);
   bool kind[2] = {false, false};  // strips, full-width strips present
   for (int i = 0; i < b->n_inst; ++i)
     kind[lbm::full_width(b->inst[i].nx, mom_nt(b), b->vec) ? 1 : 0] = true;
   cudaError_t e = cudaSuccess;
   for (int full = 0; full < 2 && e == cudaSuccess; ++full)
     if (kind[full])
-      e = lbm::launch_sweep<S>(mom_nt(b), b->vec, lbm::MODE_MOMENTS, full,
-                               (const S*)b->slab[b->cur], nullptr, b->d_inst, d_items, n, mo,
-                               b->d_status, b->stream);
+      e = lbm::launch_pair_moments(mom_nt(b), full, b->maps_mom, b->cur, b->d_inst, d_items, n, mo,
+                                   b->d_status, b->stream);
   return e;
 }
 
@@ -1235,7 +1315,7 @@ int moments_pass(Batch* b, const WorkItem* d_items, int n, MomArgs<S> mo) {
   mo.part_sum = b->d_part_sum;
   mo.part_max = b->d_part_max;
   mo.part_bad = b->d_part_bad;
-  cudaError_t e = launch_moments<S>(b, d_items, n, mo);
+  cudaError_t e = launch_moments(b, d_items, n, mo);
   if (e != cudaSuccess)
     return set_err(b->err, LBM_ECUDA, "moments kernel launch failed: %s", cudaGetErrorString(e));
   return LBM_OK;
@@ -1791,7 +1871,7 @@ int noalloc_diag_pass(Batch* b, double* part_sum, float* part_max, int* part_bad
   mo.part_max = part_max;
   mo.part_bad = part_bad;
   mo.flags = lbm::MOM_DIAG;  // no fields, no reference density
-  cudaError_t e = launch_moments<S>(b, b->d_all_items, b->n_all, mo);
+  cudaError_t e = launch_moments(b, b->d_all_items, b->n_all, mo);
   if (e != cudaSuccess)
     return set_err(b->err, LBM_ECUDA, "diagnostics pass launch failed: %s",
                    cudaGetErrorString(e));
@@ -2052,6 +2132,7 @@ int lbm_selftest_dep_timeout(lbm_handle* h, int polls) {
   if (e == cudaSuccess)
     e = lbm::launch_persist(b->rule, b->grp_nt[0],
                             b->grp_full[0] ? lbm::PERSIST_FULL : lbm::PERSIST_STRIP,
+                            b->maps_step, b->cur,
                             (float*)b->slab[b->cur], (float*)b->slab[b->cur ^ 1], b->d_inst,
                             d_items2, d_links2, 1, 2,
                             sync, sync + 1, b->d_status, 1, polls, b->shared, b->stream);
@@ -2253,8 +2334,11 @@ int lbm_save(lbm_handle* h, const char* path) {
   const InstParams& P = b->inst[0];
   const size_t bytes = 9 * (size_t)P.plane * b->esz;
   std::vector<char> buf(bytes);
-  CK(b, cudaMemcpyAsync(buf.data(), (char*)b->slab[b->cur] + P.off * b->esz, bytes,
-                        cudaMemcpyDeviceToHost, b->stream));
+  const size_t plane = (size_t)P.plane * b->esz;
+  for (int q = 0; q < lbm::Q; ++q)  // the file has the planes in the order of q
+    CK(b, cudaMemcpyAsync(buf.data() + q * plane,
+                          (char*)b->slab[b->cur] + P.off * b->esz + lbm::pos_of(q) * plane, plane,
+                          cudaMemcpyDeviceToHost, b->stream));
   CK(b, cudaStreamSynchronize(b->stream));
   FileHeader hd;
   std::memset(&hd, 0, sizeof hd);
@@ -2307,9 +2391,11 @@ int lbm_load(lbm_handle* h, const char* path) {
   uint32_t crc = crc32_update(0, &hd, sizeof hd);
   crc = crc32_update(crc, buf.data(), buf.size());
   if (crc != crc_file) return set_err(b->err, LBM_EIO, "checksum mismatch in %s", path);
+  const size_t plane = (size_t)P.plane * b->esz;
   for (int k = 0; k < 2; ++k)
-    CK(b, cudaMemcpyAsync((char*)b->slab[k] + P.off * b->esz, buf.data(), buf.size(),
-                          cudaMemcpyHostToDevice, b->stream));
+    for (int q = 0; q < lbm::Q; ++q)
+      CK(b, cudaMemcpyAsync((char*)b->slab[k] + P.off * b->esz + lbm::pos_of(q) * plane,
+                            buf.data() + q * plane, plane, cudaMemcpyHostToDevice, b->stream));
   // A state saved after full-width sweeps carries stale ghost columns; this handle's
   // tiling may sweep the lattice in strips, which read them.
   CK(b, b->fp64 ? lbm::launch_fill_ghosts<double>((double*)b->slab[b->cur], P, b->stream)

@@ -23,7 +23,7 @@ __device__ __forceinline__ long long slot_of(const InstParams& P, int q, int x, 
     }
   }
   xs = xs < 0 ? xs + P.nx : (xs >= P.nx ? xs - P.nx : xs);
-  return P.off + (long long)qs * P.plane + (long long)ys * P.pitch + GHOST + xs;
+  return P.off + (long long)pos_of(qs) * P.plane + (long long)ys * P.pitch + GHOST + xs;
 }
 
 // Refresh the ghost columns -2, -1, nx, nx+1 of every row from the columns they mirror

@@ -6,27 +6,29 @@
 
 namespace lbm {
 
-// Launch the fused sweep (MODE_STEP) or the moments/diagnostics pass (MODE_MOMENTS) over
-// n_items work items; nt (threads per CTA), vec (columns per thread) and, for the pair
-// kernel (vec 2, moments only: its steps are launch_pair), full (full-width strips, see
-// strips_for) select the instantiation.  A pair-kernel CTA whose instance is not of the
-// launched kind returns at once.
+// Launch the fused one-column sweep (MODE_STEP) or its moments/diagnostics pass
+// (MODE_MOMENTS) over n_items work items with nt threads per CTA.
 template <typename S>
-cudaError_t launch_sweep(int nt, int vec, int mode, int full, const S* fin, S* fout,
-                         const InstParams* d_inst,
+cudaError_t launch_sweep(int nt, int mode, const S* fin, S* fout, const InstParams* d_inst,
                          const WorkItem* d_items, int n_items, const MomArgs<S>& mo,
                          int* d_status, cudaStream_t st);
-// Step of the pair kernel (vec 2) for a viscosity rule (VISC_* with the constants that the
-// instances of the launch share, or PAIR_ANY).
-cudaError_t launch_pair(int rule, int nt, int full, const float* fin, float* fout,
+// Pair kernel (two columns per thread): the moments/diagnostics pass over the items of one
+// kind (full-width strips or not; a CTA whose instance is of the other kind returns at
+// once), and a step for a viscosity rule (VISC_* with the constants that the instances of the
+// launch share, or PAIR_ANY).  Both read the slab of the given index through the row maps.
+cudaError_t launch_pair_moments(int nt, int full, const RowMaps& maps, int slab,
+                                const InstParams* d_inst, const WorkItem* d_items, int n_items,
+                                const MomArgs<float>& mo, int* d_status, cudaStream_t st);
+cudaError_t launch_pair(int rule, int nt, int full, const RowMaps& maps, int slab, float* fout,
                         const InstParams* d_inst, const WorkItem* d_items, int n_items,
                         int* d_status, const PairConsts& shared, cudaStream_t st);
 template <int RULE>
-cudaError_t launch_pair_step(int nt, int full, const float* fin, float* fout,
+cudaError_t launch_pair_step(int nt, int full, const RowMaps& maps, int slab, float* fout,
                              const InstParams* d_inst, const WorkItem* d_items, int n_items,
                              int* d_status, const PairConsts& shared, cudaStream_t st);
 template <int RULE>
-cudaError_t launch_pair_persist(int nt, int kind, float* slab0, float* slab1,
+cudaError_t launch_pair_persist(int nt, int kind, const RowMaps& maps, int slab,
+                                float* slab0, float* slab1,
                                 const InstParams* d_inst, const WorkItem* items2,
                                 const ItemLink* links2, int n_items, int steps, int* queue,
                                 int* done, int* d_status, int grid, int dep_limit,
@@ -88,7 +90,8 @@ cudaError_t launch_pressure(const S* rho, const InstParams& P, double sigma, dou
 // item's kind from its instance's width).  items2 and links2 hold 2 n_items entries (the
 // even steps' list, then the odd steps'); queue (one int) and done (one int per chunk)
 // must be zero at launch; dep_limit bounds each dependency wait (DEP_WAIT_LIMIT).
-cudaError_t launch_persist(int rule, int nt, int kind, float* slab0, float* slab1,
+cudaError_t launch_persist(int rule, int nt, int kind, const RowMaps& maps, int slab,
+                           float* slab0, float* slab1,
                            const InstParams* d_inst, const WorkItem* items2,
                            const ItemLink* links2, int n_items, int steps, int* queue,
                            int* done, int* d_status, int grid, int dep_limit,
@@ -118,7 +121,7 @@ cudaError_t launch_wait_selftest(int* status, long long polls, cudaStream_t st);
 
 // Resident CTAs per SM of the step kernel instantiation (at least 1).
 template <typename S>
-int sweep_occupancy(int nt, int vec);
+int sweep_occupancy(int nt);
 
 // Whether a (storage type, threads per CTA, columns per thread) triple has a kernel.
 inline bool cfg_supported(bool fp64, int nt, int vec) {

@@ -12,19 +12,20 @@ namespace lbm {
     default: return FN<PAIR_ANY>(__VA_ARGS__);                                     \
   }
 
-cudaError_t launch_pair(int rule, int nt, int full, const float* fin, float* fout,
+cudaError_t launch_pair(int rule, int nt, int full, const RowMaps& maps, int slab, float* fout,
                         const InstParams* d_inst, const WorkItem* d_items, int n_items,
                         int* d_status, const PairConsts& shared, cudaStream_t st) {
-  LBM_BY_RULE(launch_pair_step, nt, full, fin, fout, d_inst, d_items, n_items, d_status, shared,
+  LBM_BY_RULE(launch_pair_step, nt, full, maps, slab, fout, d_inst, d_items, n_items, d_status, shared,
               st)
 }
 
-cudaError_t launch_persist(int rule, int nt, int kind, float* slab0, float* slab1,
+cudaError_t launch_persist(int rule, int nt, int kind, const RowMaps& maps, int slab,
+                           float* slab0, float* slab1,
                            const InstParams* d_inst, const WorkItem* items2,
                            const ItemLink* links2, int n_items, int steps, int* queue,
                            int* done, int* d_status, int grid, int dep_limit,
                            const PairConsts& shared, cudaStream_t st) {
-  LBM_BY_RULE(launch_pair_persist, nt, kind, slab0, slab1, d_inst, items2, links2, n_items,
+  LBM_BY_RULE(launch_pair_persist, nt, kind, maps, slab, slab0, slab1, d_inst, items2, links2, n_items,
               steps, queue, done, d_status, grid, dep_limit, shared, st)
 }
 

@@ -6,7 +6,7 @@
 namespace lbm {
 
 template <int NT, int MODE, bool FULL, int VISC>
-static cudaError_t launch_sweep2_cfg(const float* fin, float* fout, const InstParams* d_inst,
+static cudaError_t launch_sweep2_cfg(const RowMaps& maps, int slab, float* fout, const InstParams* d_inst,
                                      const WorkItem* d_items, int n_items,
                                      const MomArgs<float>& mo, int* d_status,
                                      const PairConsts& shared, cudaStream_t st) {
@@ -16,13 +16,13 @@ static cudaError_t launch_sweep2_cfg(const float* fin, float* fout, const InstPa
   if (e != cudaSuccess) return e;
   if (n_items <= 0) return cudaSuccess;
   sweep2_kernel<NT, MODE, FULL, VISC><<<n_items, NT, smem, st>>>(
-      fin, fout, d_inst, d_items, n_items, mo, d_status, shared);
+      maps, slab, fout, d_inst, d_items, n_items, mo, d_status, shared);
   return cudaGetLastError();
 }
 
 // Persistent pair kernel (sweep2_persist_kernel) with `grid` CTAs.
 template <int NT, int KIND, int VISC>
-static cudaError_t launch_persist2_cfg(float* slab0, float* slab1, const InstParams* d_inst,
+static cudaError_t launch_persist2_cfg(const RowMaps& maps, int slab, float* slab0, float* slab1, const InstParams* d_inst,
                                        const WorkItem* items2, const ItemLink* links2,
                                        int n_items, int steps, int* queue, int* done,
                                        int* d_status, int grid, int dep_limit,
@@ -33,7 +33,7 @@ static cudaError_t launch_persist2_cfg(float* slab0, float* slab1, const InstPar
   if (e != cudaSuccess) return e;
   if (n_items <= 0 || steps <= 0 || grid <= 0) return cudaSuccess;
   sweep2_persist_kernel<NT, KIND, VISC><<<grid, NT, smem, st>>>(
-      slab0, slab1, d_inst, items2, links2, n_items, steps, queue, done, d_status, dep_limit,
+      maps, slab, slab0, slab1, d_inst, items2, links2, n_items, steps, queue, done, d_status, dep_limit,
       shared);
   return cudaGetLastError();
 }
@@ -47,16 +47,16 @@ static int pair_occupancy(F* fn, int nt, size_t smem) {
 }
 
 template <int VISC>
-cudaError_t launch_pair_step(int nt, int full, const float* fin, float* fout,
+cudaError_t launch_pair_step(int nt, int full, const RowMaps& maps, int slab, float* fout,
                              const InstParams* d_inst, const WorkItem* d_items, int n_items,
                              int* d_status, const PairConsts& shared, cudaStream_t st) {
   const MomArgs<float> mo{};
 #define LBM_PAIR(T)                                                                           \
   if (nt == T)                                                                                \
-    return full ? launch_sweep2_cfg<T, MODE_STEP, true, VISC>(fin, fout, d_inst, d_items,     \
+    return full ? launch_sweep2_cfg<T, MODE_STEP, true, VISC>(maps, slab, fout, d_inst, d_items,     \
                                                               n_items, mo, d_status, shared,  \
                                                               st)                             \
-                : launch_sweep2_cfg<T, MODE_STEP, false, VISC>(fin, fout, d_inst, d_items,    \
+                : launch_sweep2_cfg<T, MODE_STEP, false, VISC>(maps, slab, fout, d_inst, d_items,    \
                                                                n_items, mo, d_status, shared, \
                                                                st);
   LBM_PAIR(32)
@@ -68,14 +68,15 @@ cudaError_t launch_pair_step(int nt, int full, const float* fin, float* fout,
 }
 
 template <int VISC>
-cudaError_t launch_pair_persist(int nt, int kind, float* slab0, float* slab1,
+cudaError_t launch_pair_persist(int nt, int kind, const RowMaps& maps, int slab,
+                                float* slab0, float* slab1,
                                 const InstParams* d_inst, const WorkItem* items2,
                                 const ItemLink* links2, int n_items, int steps, int* queue,
                                 int* done, int* d_status, int grid, int dep_limit,
                                 const PairConsts& shared, cudaStream_t st) {
 #define LBM_PERSIST_KIND(T, K)                                                               \
   if (nt == T && kind == K)                                                                  \
-    return launch_persist2_cfg<T, K, VISC>(slab0, slab1, d_inst, items2, links2, n_items,    \
+    return launch_persist2_cfg<T, K, VISC>(maps, slab, slab0, slab1, d_inst, items2, links2, n_items,    \
                                            steps, queue, done, d_status, grid, dep_limit,    \
                                            shared, st);
 #define LBM_PERSIST(T)                  \
@@ -126,12 +127,13 @@ int pair_step_occupancy(int nt) {
 }  // namespace lbm
 
 #define LBM_INSTANTIATE_PAIR(V)                                                               \
-  template cudaError_t lbm::launch_pair_step<V>(int, int, const float*, float*,               \
+  template cudaError_t lbm::launch_pair_step<V>(int, int, const lbm::RowMaps&, int, float*,               \
                                                 const lbm::InstParams*, const lbm::WorkItem*, \
                                                 int, int*, const lbm::PairConsts&,            \
                                                 cudaStream_t);                                \
   template cudaError_t lbm::launch_pair_persist<V>(                                           \
-      int, int, float*, float*, const lbm::InstParams*, const lbm::WorkItem*,                 \
+      int, int, const lbm::RowMaps&, int, float*, float*, const lbm::InstParams*,          \
+      const lbm::WorkItem*,                 \
       const lbm::ItemLink*, int, int, int*, int*, int*, int, int, const lbm::PairConsts&,     \
       cudaStream_t);                                                                          \
   template int lbm::pair_persist_occupancy<V>(int, int);                                      \

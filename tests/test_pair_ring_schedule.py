@@ -61,3 +61,31 @@ def test_four_slot_ring_schedule(nload, walls):
         if k == 1:
             phase_bit ^= 1 if o_lo else 0
             o_lo = 2 - o_lo
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_state_file_keeps_the_planes_in_velocity_order(tmp_path, precision):
+    """A state file holds plane q of the D2Q9 order as its q-th plane, whatever order the
+    planes have in device memory: uniform populations, a different value for each q."""
+    import numpy as np
+    from tests import pairs
+    c = pairs.case(21, 13, tr=0.7, sigma=0.114)
+    tw = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)
+    f = np.empty((9, 13, 21))
+    for q in range(9):
+        f[q] = tw[q] * (0.2 + 0.01 * q)
+    path = tmp_path / "state"
+    with pairs.gpu_lattice(c, precision) as L:
+        L.set_populations(f)
+        L.save(str(path))
+        L.load(str(path))
+        assert np.allclose(L.get_populations(), f, rtol=0, atol=1e-7)
+    dt = np.float64 if precision == "fp64" else np.float32
+    pitch = (21 + 16 + 7) // 8 * 8
+    n = 9 * 13 * pitch
+    raw = path.read_bytes()
+    planes = np.frombuffer(raw[-4 - n * dt().nbytes:-4], dtype=dt).reshape(9, 13, pitch)
+    inner = planes[:, :, 8:8 + 21].astype(np.float64)
+    shift = (inner - f) / tw[:, None, None]  # -rho_ref (0 in FP64), the same for every plane
+    assert np.ptp(shift) < 1e-5
