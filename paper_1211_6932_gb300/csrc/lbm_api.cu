@@ -749,12 +749,14 @@ int rebuild_items(Batch* b) {
     int rc = build_persist(b);
     if (rc) return rc;
   }
-  // Full-width strips of the pair kernel neither read nor write the ghost columns, so
-  // after steps under one set of work lists they may be stale; a pass under the new lists
-  // may use strips that read them.
-  if (!b->fp64 && b->slab[b->cur])
+  // Full-width strips neither read nor write the ghost columns, so after steps under one set
+  // of work lists they may be stale; a pass under the new lists may use strips that read
+  // them.
+  if (b->slab[b->cur])
     for (int i = 0; i < b->n_inst; ++i)
-      CK(b, lbm::launch_fill_ghosts<float>((float*)b->slab[b->cur], b->inst[i], b->stream));
+      CK(b, b->fp64
+                ? lbm::launch_fill_ghosts<double>((double*)b->slab[b->cur], b->inst[i], b->stream)
+                : lbm::launch_fill_ghosts<float>((float*)b->slab[b->cur], b->inst[i], b->stream));
   return LBM_OK;
 }
 
@@ -917,7 +919,7 @@ int launch_group(Batch* b, int g, int c, cudaStream_t st) {
   cudaError_t e;
   if (b->fp64) {
     MomArgs<double> mo{};
-    e = lbm::launch_sweep<double>(b->grp_nt[g], lbm::MODE_STEP, (const double*)b->slab[c],
+    e = lbm::launch_sweep<double>(b->grp_nt[g], lbm::MODE_STEP, b->grp_full[g], (const double*)b->slab[c],
                                   (double*)b->slab[c ^ 1], b->d_inst, items, n, mo, b->d_status,
                                   st);
   } else if (b->vec == 2) {
@@ -925,7 +927,7 @@ int launch_group(Batch* b, int g, int c, cudaStream_t st) {
                          (float*)b->slab[c ^ 1], b->d_inst, items, n, b->d_status, b->shared, st);
   } else {
     MomArgs<float> mo{};
-    e = lbm::launch_sweep<float>(b->grp_nt[g], lbm::MODE_STEP, (const float*)b->slab[c],
+    e = lbm::launch_sweep<float>(b->grp_nt[g], lbm::MODE_STEP, b->grp_full[g], (const float*)b->slab[c],
                                  (float*)b->slab[c ^ 1], b->d_inst, items, n, mo, b->d_status, st);
   }
   if (e != cudaSuccess)
@@ -1286,26 +1288,26 @@ int get_pops(Batch* b, int i, double* f) {
 }
 
 // Launch the moments/diagnostics kernel over a device list of n items on the batch's
-// stream.  The pair kernel has strip and full-width instantiations: both are launched over
+// stream.  The kernels have strip and full-width instantiations: both are launched over
 // the whole list, and each CTA works only on an item of its own kind.
-cudaError_t launch_moments(const Batch* b, const WorkItem* d_items, int n,
-                           const MomArgs<double>& mo) {
-  return lbm::launch_sweep<double>(mom_nt(b), lbm::MODE_MOMENTS, (const double*)b->slab[b->cur],
-                                   nullptr, b->d_inst, d_items, n, mo, b->d_status, b->stream);
-}
-cudaError_t launch_moments(const Batch* b, const WorkItem* d_items, int n,
-                           const MomArgs<float>& mo) {
-  if (b->vec != 2)
-    return lbm::launch_sweep<float>(mom_nt(b), lbm::MODE_MOMENTS, (const float*)b->slab[b->cur],
-                                    nullptr, b->d_inst, d_items, n, mo, b->d_status, b->stream);
+template <typename S>
+cudaError_t launch_moments(const Batch* b, const WorkItem* d_items, int n, const MomArgs<S>& mo) {
   bool kind[2] = {false, false};  // strips, full-width strips present
   for (int i = 0; i < b->n_inst; ++i)
     kind[lbm::full_width(b->inst[i].nx, mom_nt(b), b->vec) ? 1 : 0] = true;
   cudaError_t e = cudaSuccess;
-  for (int full = 0; full < 2 && e == cudaSuccess; ++full)
-    if (kind[full])
-      e = lbm::launch_pair_moments(mom_nt(b), full, b->maps_mom, b->cur, b->d_inst, d_items, n, mo,
-                                   b->d_status, b->stream);
+  for (int full = 0; full < 2 && e == cudaSuccess; ++full) {
+    if (!kind[full]) continue;
+    if constexpr (sizeof(S) == 4) {
+      if (b->vec == 2) {
+        e = lbm::launch_pair_moments(mom_nt(b), full, b->maps_mom, b->cur, b->d_inst, d_items, n,
+                                     mo, b->d_status, b->stream);
+        continue;
+      }
+    }
+    e = lbm::launch_sweep<S>(mom_nt(b), lbm::MODE_MOMENTS, full, (const S*)b->slab[b->cur], nullptr,
+                             b->d_inst, d_items, n, mo, b->d_status, b->stream);
+  }
   return e;
 }
 

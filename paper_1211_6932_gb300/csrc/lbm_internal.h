@@ -7,9 +7,11 @@
 namespace lbm {
 
 // Launch the fused one-column sweep (MODE_STEP) or its moments/diagnostics pass
-// (MODE_MOMENTS) over n_items work items with nt threads per CTA.
+// (MODE_MOMENTS) over n_items work items with nt threads per CTA, in full-width strips or not
+// (see strips_for; a CTA of the moments pass whose instance is of the other kind returns at
+// once).
 template <typename S>
-cudaError_t launch_sweep(int nt, int mode, const S* fin, S* fout, const InstParams* d_inst,
+cudaError_t launch_sweep(int nt, int mode, int full, const S* fin, S* fout, const InstParams* d_inst,
                          const WorkItem* d_items, int n_items, const MomArgs<S>& mo,
                          int* d_status, cudaStream_t st);
 // Pair kernel (two columns per thread): the moments/diagnostics pass over the items of one
@@ -132,11 +134,11 @@ inline bool cfg_supported(bool fp64, int nt, int vec) {
 
 // Columns owned by one CTA of a configuration.
 inline int strip_width(int nt, int vec) { return vec == 2 ? 2 * nt - 4 : nt - 4; }
-// CTA strips across an instance of nx columns.  The pair kernel (vec 2) covers an
-// instance with nx <= 2 nt in one full-width strip: every thread owns two columns, the
-// periodic wrap in x is taken inside shared memory and the ghost columns are neither
-// read nor written.  Otherwise strips of strip_width owned columns.
-inline bool full_width(int nx, int nt, int vec) { return vec == 2 && nx <= 2 * nt; }
+// CTA strips across an instance of nx columns.  An instance with nx <= nt * vec is covered
+// in one full-width strip: every thread owns its columns, the periodic wrap in x is taken
+// inside shared memory and the ghost columns are neither read nor written.  Otherwise strips
+// of strip_width owned columns.
+inline bool full_width(int nx, int nt, int vec) { return nx <= nt * vec; }
 inline int strips_for(int nx, int nt, int vec) {
   if (full_width(nx, nt, vec)) return 1;
   const int W = strip_width(nt, vec);

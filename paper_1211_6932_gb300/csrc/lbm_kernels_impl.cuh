@@ -22,39 +22,43 @@ static cudaError_t ensure_smem_attr(F* fn, size_t smem, std::atomic<unsigned lon
   return e;
 }
 
-template <typename S, int NT, int MODE>
+template <typename S, int NT, int MODE, bool FULL>
 static cudaError_t launch_sweep_cfg(const S* fin, S* fout, const InstParams* d_inst,
                                     const WorkItem* d_items, int n_items, const MomArgs<S>& mo,
                                     int* d_status, cudaStream_t st) {
   constexpr size_t smem = SweepCfg<S, NT>::BYTES;
   static std::atomic<unsigned long long> done{0};
-  cudaError_t e = ensure_smem_attr(sweep_kernel<S, NT, MODE>, smem, done);
+  cudaError_t e = ensure_smem_attr(sweep_kernel<S, NT, MODE, FULL>, smem, done);
   if (e != cudaSuccess) return e;
   if (n_items <= 0) return cudaSuccess;
-  sweep_kernel<S, NT, MODE><<<n_items, NT, smem, st>>>(fin, fout, d_inst, d_items, n_items,
+  sweep_kernel<S, NT, MODE, FULL><<<n_items, NT, smem, st>>>(fin, fout, d_inst, d_items, n_items,
                                                        mo, d_status);
   return cudaGetLastError();
 }
 
 template <typename S, int NT>
-static cudaError_t launch_sweep_mode(int mode, const S* fin, S* fout, const InstParams* d_inst,
+static cudaError_t launch_sweep_mode(int mode, int full, const S* fin, S* fout, const InstParams* d_inst,
                                      const WorkItem* d_items, int n_items,
                                      const MomArgs<S>& mo, int* d_status, cudaStream_t st) {
   if (mode == MODE_STEP)
-    return launch_sweep_cfg<S, NT, MODE_STEP>(fin, fout, d_inst, d_items, n_items, mo,
-                                              d_status, st);
-  return launch_sweep_cfg<S, NT, MODE_MOMENTS>(fin, fout, d_inst, d_items, n_items, mo,
-                                               d_status, st);
+    return full ? launch_sweep_cfg<S, NT, MODE_STEP, true>(fin, fout, d_inst, d_items, n_items,
+                                                           mo, d_status, st)
+                : launch_sweep_cfg<S, NT, MODE_STEP, false>(fin, fout, d_inst, d_items, n_items,
+                                                            mo, d_status, st);
+  return full ? launch_sweep_cfg<S, NT, MODE_MOMENTS, true>(fin, fout, d_inst, d_items, n_items,
+                                                            mo, d_status, st)
+              : launch_sweep_cfg<S, NT, MODE_MOMENTS, false>(fin, fout, d_inst, d_items, n_items,
+                                                             mo, d_status, st);
 }
 
 template <typename S, int NT>
 static int occupancy_cfg() {
   constexpr size_t smem = SweepCfg<S, NT>::BYTES;
-  cudaFuncSetAttribute(sweep_kernel<S, NT, MODE_STEP>,
+  cudaFuncSetAttribute(sweep_kernel<S, NT, MODE_STEP, false>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int occ = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &occ, sweep_kernel<S, NT, MODE_STEP>, NT, smem);
+      &occ, sweep_kernel<S, NT, MODE_STEP, false>, NT, smem);
   return (e == cudaSuccess && occ > 0) ? occ : 1;
 }
 
