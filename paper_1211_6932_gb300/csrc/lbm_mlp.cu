@@ -18,6 +18,14 @@
 //                     parameters more than 1e-5 from the oracle's, against 1 % allowed:
 //                     the summation order moves parameters whose second moment is tiny.)
 // Runs of training updates are replayed from a captured CUDA graph.
+//
+// An update is a chain of latencies, not work: 256 rows are 7 MFLOP.  Both kernels are
+// launched as programmatic dependents, so that a kernel's launch and whatever does not need
+// its predecessor's results overlap the predecessor; a block has two rows, so that 256 rows
+// use 128 SMs and two warps share a block's shared-memory reads instead of eight; weights are
+// staged with 16-byte loads issued together; the bias corrections and the loss have a warp and
+// a block of their own.  256 rows: 18.9 us an update before, 7.3 now, with the same sums in
+// the same order.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -38,9 +46,9 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + NH * NI, OFF_W2 = OFF_B1 + NH,
 static_assert(OFF_B3 + NO == NP, "parameter packing");
 constexpr int W1S = NI + 1;  // padded row strides in shared memory
 constexpr int W2S = NH + 1;
-constexpr int ROWS_PER_BLOCK = 8;  // warps per block in the rows kernel
-constexpr int PARAM_THREADS = 256;
-constexpr int PARAM_SLICES = PARAM_THREADS / 32;  // row slices (warps) per parameter
+constexpr int ROWS_PER_BLOCK = 2;  // warps per block in the rows kernel
+constexpr int PARAM_SLICES = 8;    // row slices (warps) per parameter
+constexpr int PARAM_THREADS = 32 * PARAM_SLICES;
 constexpr int PARAM_BLOCKS = (NP + 31) / 32;      // 32 parameters per block
 constexpr int kGraphUpdates = 50;
 constexpr int kLossHistory = 1 << 16;
@@ -79,6 +87,15 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// Programmatic dependent launch: wait until the preceding kernel of the stream has completed
+// (nothing to wait for after an ordinary launch), and let the following one be launched.
+__device__ __forceinline__ void wait_predecessor() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 enum { ROWS_PREDICT = 0, ROWS_TRAIN = 1 };
 
 template <int MODE>
@@ -89,25 +106,62 @@ __global__ void __launch_bounds__(ROWS_PER_BLOCK * 32) mlp_rows_kernel(
   __shared__ float sW1[NH * W1S], sB1[NH], sW2[NH * W2S], sB2[NH], sW3[NO * NH], sB3[NO];
   __shared__ float sBuf[ROWS_PER_BLOCK][NH];
   const int tid = threadIdx.x;
-  for (int i = tid; i < NP; i += blockDim.x) {
-    const float v = __bfloat162float(w[i]);
-    if (i < OFF_B1) sW1[(i / NI) * W1S + i % NI] = v;
-    else if (i < OFF_W2) sB1[i - OFF_B1] = v;
-    else if (i < OFF_B2) sW2[((i - OFF_W2) / NH) * W2S + (i - OFF_W2) % NH] = v;
-    else if (i < OFF_W3) sB2[i - OFF_B2] = v;
-    else if (i < OFF_B3) sW3[i - OFF_W3] = v;
-    else sB3[i - OFF_B3] = v;
-  }
-  __syncthreads();
-  if (MODE == ROWS_TRAIN && update_counter && blockIdx.x == 0 && tid == 0) ++*update_counter;
   const int warp = tid >> 5, lane = tid & 31;
   const int row = blockIdx.x * ROWS_PER_BLOCK + warp;
+  float xn[NI], tn[NO];
+  if (row < n) {
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+      xn[i] = (x[(size_t)row * NI + i] - sc.in_mean[i]) / sc.in_scale[i];
+    if (MODE == ROWS_TRAIN)
+#pragma unroll
+      for (int o = 0; o < NO; ++o)
+        tn[o] = (t[(size_t)row * NO + o] - sc.out_mean[o]) / sc.out_scale[o];
+  }
+  wait_predecessor();  // the weights of the last update; everything above is constant
+  // the weights in groups of eight, which the packing keeps within one array each
+  static_assert(OFF_B1 % 8 == 0 && OFF_W2 % 8 == 0 && OFF_B2 % 8 == 0 && OFF_W3 % 8 == 0 &&
+                    OFF_B3 % 8 == 0 && NH % 8 == 0 && 8 % NI == 0,
+                "groups of eight weights");
+  constexpr int GROUPS = OFF_B3 / 8, PER = (GROUPS + ROWS_PER_BLOCK * 32 - 1) / (ROWS_PER_BLOCK * 32);
+  uint4 v[PER];
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int g = tid + k * ROWS_PER_BLOCK * 32;
+    if (g < GROUPS) v[k] = reinterpret_cast<const uint4*>(w)[g];
+  }
+  if (tid < NO) sB3[tid] = __bfloat162float(w[OFF_B3 + tid]);
+  if (MODE == ROWS_TRAIN && update_counter && blockIdx.x == 0 && tid == 0) ++*update_counter;
+  launch_dependents();
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int i = (tid + k * ROWS_PER_BLOCK * 32) * 8;
+    if (i >= OFF_B3) continue;
+    float f[8];
+    const __nv_bfloat162* h2v = reinterpret_cast<const __nv_bfloat162*>(&v[k]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 p2 = __bfloat1622float2(h2v[e]);
+      f[2 * e] = p2.x;
+      f[2 * e + 1] = p2.y;
+    }
+    if (i >= OFF_W2 && i < OFF_B2) {
+      float* d = sW2 + ((i - OFF_W2) / NH) * W2S + (i - OFF_W2) % NH;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) d[e] = f[e];
+    } else if (i < OFF_B1) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) sW1[((i + e) / NI) * W1S + (i + e) % NI] = f[e];
+    } else {
+      float* d = i < OFF_W2 ? sB1 + (i - OFF_B1) : i < OFF_W3 ? sB2 + (i - OFF_B2)
+                                                             : sW3 + (i - OFF_W3);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) d[e] = f[e];
+    }
+  }
+  __syncthreads();
   if (row >= n) return;
   float* buf = sBuf[warp];
-
-  float xn[NI];
-#pragma unroll
-  for (int i = 0; i < NI; ++i) xn[i] = (x[(size_t)row * NI + i] - sc.in_mean[i]) / sc.in_scale[i];
 
   // layer 1
   float z1[2], h1[2];
@@ -157,8 +211,7 @@ __global__ void __launch_bounds__(ROWS_PER_BLOCK * 32) mlp_rows_kernel(
   float dy[NO], l2 = 0.f;
 #pragma unroll
   for (int o = 0; o < NO; ++o) {
-    const float tn = (t[(size_t)row * NO + o] - sc.out_mean[o]) / sc.out_scale[o];
-    const float e = y[o] - tn;
+    const float e = y[o] - tn[o];
     l2 = fmaf(e, e, l2);
     dy[o] = inv * e;
   }
@@ -212,18 +265,22 @@ __global__ void __launch_bounds__(ROWS_PER_BLOCK * 32) mlp_rows_kernel(
 
 enum { PARAM_GRAD = 0, PARAM_ADAM = 1 };
 
-__global__ void __launch_bounds__(PARAM_THREADS) mlp_param_kernel(
+__global__ void __launch_bounds__(PARAM_THREADS + 32) mlp_param_kernel(
     RowBufs rb, int n, float* __restrict__ master, __nv_bfloat16* __restrict__ w,
     float* __restrict__ m1, float* __restrict__ m2, float* __restrict__ grad_out, AdamArgs a,
     int mode, const long long* __restrict__ update_counter, float* __restrict__ loss_hist,
     float* __restrict__ loss_out) {
   const int tid = threadIdx.x;
-  if (blockIdx.x == 0) {
+  if (blockIdx.x == PARAM_BLOCKS) {
     // loss: fixed partition of the rows over the threads, then a fixed tree
     __shared__ float red[PARAM_THREADS];
-    float s = 0.f;
-    for (int r = tid; r < n; r += PARAM_THREADS) s += rb.lrow[r];
-    red[tid] = s;
+    wait_predecessor();
+    launch_dependents();
+    if (tid < PARAM_THREADS) {
+      float s = 0.f;
+      for (int r = tid; r < n; r += PARAM_THREADS) s += rb.lrow[r];
+      red[tid] = s;
+    }
     __syncthreads();
     for (int h = PARAM_THREADS / 2; h > 0; h >>= 1) {
       if (tid < h) red[tid] += red[tid + h];
@@ -235,10 +292,20 @@ __global__ void __launch_bounds__(PARAM_THREADS) mlp_param_kernel(
       if (mode == PARAM_ADAM && loss_hist)
         loss_hist[(*update_counter - 1) & (kLossHistory - 1)] = L;
     }
+    return;
   }
   const int lane = tid & 31, slice = tid >> 5;
   const int p = blockIdx.x * 32 + lane;
   __shared__ float part[PARAM_SLICES][32];
+  __shared__ float bias1, bias2;  // 1 - beta^k
+  // the last update's moments and weight: that kernel has completed before this one's
+  // predecessor lets it be launched
+  float old1 = 0.f, old2 = 0.f, oldw = 0.f;
+  if (slice == 0 && p < NP && mode == PARAM_ADAM) {
+    old1 = m1[p];
+    old2 = m2[p];
+    oldw = master[p];
+  }
   // dL/dp = sum over rows of (delta of the output unit) x (input value): warp `slice` sums
   // rows slice, slice + PARAM_SLICES, ... in order, lane l for parameter p
   const float* da = nullptr;
@@ -257,32 +324,41 @@ __global__ void __launch_bounds__(PARAM_THREADS) mlp_param_kernel(
   } else {
     da = rb.dy; sa = NO; ia = p - OFF_B3;
   }
-  float g = 0.f;
-  if (p < NP) {
-    if (xb) {
-#pragma unroll 4
-      for (int r = slice; r < n; r += PARAM_SLICES)
-        g = fmaf(da[(size_t)r * sa + ia], xb[(size_t)r * sb + ib], g);
-    } else {
-#pragma unroll 4
-      for (int r = slice; r < n; r += PARAM_SLICES) g += da[(size_t)r * sa + ia];
+  wait_predecessor();
+  launch_dependents();
+  if (slice == PARAM_SLICES) {  // the last warp: Adam's bias corrections meanwhile
+    if (mode == PARAM_ADAM && lane < 2) {
+      const float k = (float)*update_counter;
+      const float c = 1.f - powf(lane ? a.beta2 : a.beta1, k);
+      (lane ? bias2 : bias1) = c;
     }
+  } else {
+    float g = 0.f;
+    if (p < NP) {
+      if (xb) {
+#pragma unroll 16
+        for (int r = slice; r < n; r += PARAM_SLICES)
+          g = fmaf(da[(size_t)r * sa + ia], xb[(size_t)r * sb + ib], g);
+      } else {
+#pragma unroll 16
+        for (int r = slice; r < n; r += PARAM_SLICES) g += da[(size_t)r * sa + ia];
+      }
+    }
+    part[slice][lane] = g;
   }
-  part[slice][lane] = g;
   __syncthreads();
   if (slice != 0 || p >= NP) return;
-  g = part[0][lane];
+  float g = part[0][lane];
 #pragma unroll
   for (int k = 1; k < PARAM_SLICES; ++k) g += part[k][lane];
   if (grad_out) grad_out[p] = g;
   if (mode != PARAM_ADAM) return;
   // Adam (Kingma & Ba 2015, Algorithm 1) on the FP32 master weight
-  const float k = (float)*update_counter;
-  const float mm = fmaf(a.beta1, m1[p], (1.f - a.beta1) * g);
-  const float vv = fmaf(a.beta2, m2[p], (1.f - a.beta2) * g * g);
-  const float mhat = mm / (1.f - powf(a.beta1, k));
-  const float vhat = vv / (1.f - powf(a.beta2, k));
-  const float pm = master[p] - a.lr * mhat / (sqrtf(vhat) + a.eps);
+  const float mm = fmaf(a.beta1, old1, (1.f - a.beta1) * g);
+  const float vv = fmaf(a.beta2, old2, (1.f - a.beta2) * g * g);
+  const float mhat = mm / bias1;
+  const float vhat = vv / bias2;
+  const float pm = oldw - a.lr * mhat / (sqrtf(vhat) + a.eps);
   m1[p] = mm;
   m2[p] = vv;
   master[p] = pm;
@@ -366,12 +442,28 @@ void free_all(lbm_mlp* h) {
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
 }
 
+// Launch as a programmatic dependent of the stream's previous kernel.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), int blocks, int threads, cudaStream_t st,
+                             A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 int launch_rows(lbm_mlp* h, int mode, int n, double* y_out, long long* counter,
                 cudaStream_t st) {
   const int blocks = (n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK;
   if (mode == ROWS_TRAIN)
-    mlp_rows_kernel<ROWS_TRAIN><<<blocks, ROWS_PER_BLOCK * 32, 0, st>>>(h->w, h->x, h->t, n, h->sc,
-                                                                       h->rb, y_out, counter);
+    MCK(h, launch_dependent(mlp_rows_kernel<ROWS_TRAIN>, blocks, ROWS_PER_BLOCK * 32, st, h->w,
+                            h->x, h->t, n, h->sc, h->rb, y_out, counter));
   else
     mlp_rows_kernel<ROWS_PREDICT><<<blocks, ROWS_PER_BLOCK * 32, 0, st>>>(
         h->w, h->xp, nullptr, n, h->sc, h->rb, y_out, counter);
@@ -382,10 +474,9 @@ int launch_rows(lbm_mlp* h, int mode, int n, double* y_out, long long* counter,
 int launch_update(lbm_mlp* h, const AdamArgs& a, cudaStream_t st) {
   int rc = launch_rows(h, ROWS_TRAIN, h->n, nullptr, h->counter, st);
   if (rc) return rc;
-  mlp_param_kernel<<<PARAM_BLOCKS, PARAM_THREADS, 0, st>>>(
-      h->rb, h->n, h->master, h->w, h->m1, h->m2, nullptr, a, PARAM_ADAM, h->counter,
-      h->loss_hist, nullptr);
-  MCK(h, cudaGetLastError());
+  MCK(h, launch_dependent(mlp_param_kernel, PARAM_BLOCKS + 1, PARAM_THREADS + 32, st, h->rb, h->n,
+                          h->master, h->w, h->m1, h->m2, (float*)nullptr, a, (int)PARAM_ADAM,
+                          h->counter, h->loss_hist, (float*)nullptr));
   return LBM_OK;
 }
 
@@ -599,12 +690,14 @@ int lbm_mlp_train(lbm_mlp* h, int steps, const lbm_adam* opt, float* losses) {
   MCK(h, cudaStreamSynchronize(h->stream));
   if (losses && steps > 0) {
     // losses of updates start+1 .. start+steps live at (index - 1) mod the history size
-    std::vector<float> hist(kLossHistory);
-    MCK(h, cudaMemcpy(hist.data(), h->loss_hist, kLossHistory * sizeof(float),
-                      cudaMemcpyDeviceToHost));
-    for (int k = 0; k < steps; ++k) {
-      const long long idx = start + k;
-      losses[k] = (steps - k <= kLossHistory) ? hist[idx & (kLossHistory - 1)] : NAN;
+    int k = 0;
+    for (; steps - k > kLossHistory; ++k) losses[k] = NAN;
+    while (k < steps) {  // up to the end of the history, then from its start
+      const int at = (int)((start + k) & (kLossHistory - 1));
+      const int m = std::min(steps - k, kLossHistory - at);
+      MCK(h, cudaMemcpy(losses + k, h->loss_hist + at, m * sizeof(float),
+                        cudaMemcpyDeviceToHost));
+      k += m;
     }
   }
   return LBM_OK;
@@ -616,7 +709,7 @@ int lbm_mlp_gradient(lbm_mlp* h, float* grad, float* loss) {
   MlpDeviceGuard guard(h);
   int rc = launch_rows(h, ROWS_TRAIN, h->n, nullptr, nullptr, h->stream);
   if (rc) return rc;
-  mlp_param_kernel<<<PARAM_BLOCKS, PARAM_THREADS, 0, h->stream>>>(
+  mlp_param_kernel<<<PARAM_BLOCKS + 1, PARAM_THREADS + 32, 0, h->stream>>>(
       h->rb, h->n, h->master, h->w, h->m1, h->m2, h->grad, AdamArgs{}, PARAM_GRAD, nullptr,
       nullptr, h->loss_one);
   MCK(h, cudaGetLastError());
