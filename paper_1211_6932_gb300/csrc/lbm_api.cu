@@ -102,6 +102,8 @@ struct Batch {
   bool own_stream = false;
   cudaStream_t cap_stream = nullptr;
   int nt = 0, vec = 0, rows_req = 0, rows = 0;  // threads and columns/thread per CTA, rows per sweep
+  bool nt_auto = false;  // a single lattice whose CTA width is chosen with its chunk height
+  int mom_rows = 0;      // chunk height of the moments/diagnostics pass
   // Step launches: group g runs items [grp_begin[g], grp_begin[g+1]) with grp_nt[g]
   // threads, in full-width strips if grp_full[g] (pair kernel).  One group per kernel
   // width (one width, unless nt == LBM_TILE_PER_INSTANCE: then each instance has the width
@@ -343,7 +345,9 @@ bool tiling_ok(bool fp64, int nt, int vec) {
 }
 
 // Threads per CTA of the moments/diagnostics pass (one uniform tiling over all instances).
-int mom_nt(const Batch* b) { return per_instance(b) ? 128 : b->nt; }
+int mom_nt(const Batch* b) {
+  return per_instance(b) ? 128 : b->nt_auto ? default_threads(b->fp64) : b->nt;
+}
 
 constexpr int kPairThreads[Batch::kMaxWidths] = {32, 64, 96, 128};
 constexpr int kRowFixedCols = 57;  // per-row work of a strip row, in computed columns
@@ -475,6 +479,92 @@ int default_rows(const Batch* b) {
   return r6;
 }
 
+// CTA width and chunk height of a single lattice stepped with one launch per step, from a
+// model of the step's time: the time of a step alone on the GPU plus its work, the SM time of
+// all its CTAs, since lattices of a study often share the GPU.
+//
+// FP32 pair kernel, in us (fitted to 18 sizes from 64 x 64 to 1740 x 718, four widths and 14
+// heights, within 10 %): 2.4 for the launch and the first row, then per row (and one more of
+// start-up) a latency and the issue of the W warps that the busiest SM holds; with more items
+// than resident CTAs, the work itself.  Chunks used to be eight rows at least: 64 x 64 stepped
+// in 7.4 us and takes 3.4 with one-row chunks, 601 x 407 in 9.6 and 6.9, and 1024^2 in 17.2
+// (strips of 252 columns cover 1260) and 14.7 (six of 188 cover 1128).
+struct Tiling {
+  int nt, rows;
+};
+Tiling choose_pair_tiling(const Batch* b, const std::vector<int>& widths) {
+  const InstParams& P = b->inst[0];
+  const int sms = std::max(b->sms, 1);
+  Tiling best{widths[0], 8};
+  double best_cost = -1.0;
+  for (int nt : widths) {
+    const int occ = lbm::pair_occupancy(b->rule, nt);
+    const long long strips = lbm::strips_for(P.nx, nt, 2);
+    const double w = nt / 32.0, latency = lbm::full_width(P.nx, nt, 2) ? 0.40 : 0.62;
+    for (int rows = 1; rows <= 64; ++rows) {
+      const long long items = strips * ((P.ny + rows - 1) / rows);
+      const long long k = (items + sms - 1) / sms;
+      const double work = items * w * (rows + 1.5) * 0.0795 / sms;
+      const double row = latency + 0.05 * std::min<long long>(k, occ) * w;
+      const double alone = 2.4 + (k <= occ ? (rows + 1) * row : work + 0.1 * (rows + 1) * row);
+      if (best_cost < 0 || alone + work < best_cost) {
+        best_cost = alone + work;
+        best = {nt, rows};
+      }
+    }
+  }
+  return best;
+}
+
+// FP64, whose kernel is bound by the FP64 pipe: a row of a 64-thread CTA keeps an SM's pipe
+// for 2.4 us (and takes 5.2 alone), a chunk costs its rows and 0.73 of one for the psi of its
+// halo rows.  128^2 runs in 11.5 us a step with one full-width CTA of 128 a row (14.9 with
+// strips of 60), 500 x 400 in 68 with 64 x 6 (116 with 128 x 4).
+Tiling choose_fp64_tiling(const Batch* b, const std::vector<int>& widths) {
+  const InstParams& P = b->inst[0];
+  const int sms = std::max(b->sms, 1);
+  Tiling best{widths[0], 1};
+  double best_cost = -1.0;
+  for (int nt : widths) {
+    const int occ = lbm::sweep_occupancy<double>(nt);
+    const long long strips = lbm::strips_for(P.nx, nt, 1);
+    const double w = nt / 64.0;
+    for (int rows = 1; rows <= 64; ++rows) {
+      const long long items = strips * ((P.ny + rows - 1) / rows);
+      const long long k = (items + sms - 1) / sms;
+      const double re = rows + 0.73;
+      const double cost = k <= occ ? re * std::max(5.2, 2.4 * k * w)
+                                   : items * re * 2.4 * w / sms + 1.2 * 5.2 * re;
+      if (best_cost < 0 || cost < best_cost) {
+        best_cost = cost;
+        best = {nt, rows};
+      }
+    }
+  }
+  return best;
+}
+
+// Sets the chunk height, and the CTA width where that is free, from the requests.  The
+// moments pass keeps the default width and height, so the order of its sums, and with it
+// the last bits of the diagnostics, does not depend on how a lattice is stepped.
+void choose_tiling(Batch* b) {
+  if (b->nt_auto) b->nt = default_threads(b->fp64);
+  b->rows = b->mom_rows = b->rows_req > 0 ? b->rows_req : default_rows(b);
+  if (b->rows_req > 0 || b->n_inst != 1 || per_instance(b) || !b->active[0]) return;
+  if (b->fp64) {
+    const Tiling t = choose_fp64_tiling(
+        b, b->nt_auto ? std::vector<int>{128, 64} : std::vector<int>{b->nt});
+    b->nt = t.nt;
+    b->rows = t.rows;
+  } else if (b->vec == 2 && persist_env() != 2 &&
+             !(persist_allowed(b) && persist_items_ok(b, b->rows))) {
+    const Tiling t = choose_pair_tiling(
+        b, b->nt_auto ? std::vector<int>{128, 96, 64, 32} : std::vector<int>{b->nt});
+    b->nt = t.nt;
+    b->rows = t.rows;
+  }
+}
+
 // Work items of instance i: strips of W owned columns by chunks of `rows` rows.
 void append_items(const InstParams& P, int i, int nt, int vec, int rows,
                   std::vector<WorkItem>& out) {
@@ -522,7 +612,7 @@ void make_all_items(const Batch* b, std::vector<WorkItem>& out, std::vector<int>
   out.clear();
   begin.assign(1, 0);
   for (int i = 0; i < b->n_inst; ++i) {
-    append_items(b->inst[i], i, mom_nt(b), b->vec, b->rows, out);
+    append_items(b->inst[i], i, mom_nt(b), b->vec, b->mom_rows, out);
     begin.push_back((int)out.size());
   }
 }
@@ -708,11 +798,11 @@ int rebuild_items(Batch* b) {
     b->inst_nt.resize(b->n_inst);
     for (int i = 0; i < b->n_inst; ++i) b->inst_nt[i] = pair_threads_for(b->inst[i].nx);
   }
+  choose_tiling(b);
   {
     int rc = build_maps(b);
     if (rc) return rc;
   }
-  b->rows = b->rows_req > 0 ? b->rows_req : default_rows(b);
   make_step_items(b);
   make_all_items(b, b->all_items, b->item_begin);
   b->n_items = (int)b->items.size();
@@ -872,6 +962,7 @@ int create_batch(Batch* b, int n, const lbm_instance* in, bool fp64, int psi_fp6
   b->dense_elems = dense;
   set_rule(b);
   b->nt = nt_;
+  b->nt_auto = nt == 0 && n == 1 && vec_ == default_vec(fp64);
   b->vec = vec_;
   b->rows_req = rows;
   int dev_count = 0;
@@ -1686,6 +1777,7 @@ int apply_tiling(Batch* b, int nt, int vec, int rows, bool persist = true) {
   if (!tiling_ok(b->fp64, nt, vec))
     return set_err(b->err, LBM_EINVAL, "tiling %d threads x %d columns not available", nt, vec);
   b->nt = nt;
+  b->nt_auto = false;
   b->vec = vec;
   b->rows_req = rows;
   b->persist_off = !persist;
@@ -2305,6 +2397,7 @@ int lbm_set_tiling(lbm_handle* h, int threads, int vec, int rows) {
                    vec_);
   if (rows < 0) return set_err(b->err, LBM_EINVAL, "tile_rows must be >= 0");
   b->nt = nt_;
+  b->nt_auto = threads == 0 && vec_ == default_vec(b->fp64);
   b->vec = vec_;
   b->rows_req = rows;
   b->persist_off = false;

@@ -1,0 +1,31 @@
+"""Every tiling of the pair kernel gives the same bits (the arithmetic of a node does not
+depend on the CTA that computes it), so the default tiling of small and ragged lattices,
+with chunks down to one row, is compared with chunks of eight rows of 128-thread CTAs: full
+width and strips, even and odd widths (ghost columns written as pairs and one by one), a last
+strip of one column or of two, walls."""
+import numpy as np
+import pytest
+
+from tests import pairs
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(1, 1), (2, 5), (7, 3), (64, 64), (65, 40), (66, 9), (125, 33), (126, 20), (193, 147),
+         (253, 21), (257, 30), (300, 17), (601, 47)]
+
+
+@pytest.mark.parametrize("walls", [False, True])
+def test_default_tiling_equals_eight_row_chunks(walls):
+    for k, (nx, ny) in enumerate(SIZES):
+        c = pairs.case(nx, ny, tr=0.75, sigma=0.114, walls=walls, visc="step", nu_l=0.05,
+                       nu_v=0.3)
+        f = pairs.droplet_state(c, vel=0.02, seed=k)
+        got = []
+        for kw in ({}, {"tile_threads": 128, "tile_rows": 8}, {"tile_threads": 32, "tile_rows": 1},
+                   {"tile_threads": 64, "tile_rows": 3}):
+            with pairs.gpu_lattice(c, "fp32", **kw) as L:
+                L.set_populations(f)
+                L.step(70)
+                got.append(L.get_populations())
+        for g in got[1:]:
+            assert np.array_equal(got[0], g), (nx, ny)
