@@ -34,7 +34,8 @@ using lbm::WorkItem;
 
 namespace {
 
-constexpr int kGraphSteps = 64;  // even, so a replay returns to the same slab
+constexpr int kGraphLog = 6;
+constexpr int kGraphSteps = 1 << kGraphLog;  // even, so a replay returns to the same slab
 thread_local std::string g_thread_err;
 
 struct Batch {
@@ -104,6 +105,7 @@ struct Batch {
   int nt = 0, vec = 0, rows_req = 0, rows = 0;  // threads and columns/thread per CTA, rows per sweep
   bool nt_auto = false;  // a single lattice whose CTA width is chosen with its chunk height
   int mom_rows = 0;      // chunk height of the moments/diagnostics pass
+  bool dependent = false;  // steps are launched as programmatic dependents (overlap_ok)
   // Step launches: group g runs items [grp_begin[g], grp_begin[g+1]) with grp_nt[g]
   // threads, in full-width strips if grp_full[g] (pair kernel).  One group per kernel
   // width (one width, unless nt == LBM_TILE_PER_INSTANCE: then each instance has the width
@@ -117,7 +119,10 @@ struct Batch {
   int grp_begin[kMaxGroups + 1] = {};
   cudaStream_t grp_stream[kMaxGroups - 1] = {};  // graph branches
   cudaEvent_t grp_fork = nullptr, grp_join[kMaxGroups - 1] = {};
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  // Graphs of 2^k steps from either slab (kGraphSteps = 2^kGraphLog), and how often a run of
+  // that many steps has been queued launch by launch.
+  cudaGraphExec_t graph[kGraphLog + 1][2] = {};
+  int graph_uses[kGraphLog + 1][2] = {};
   // Buffers allocated with guard bands (lbm_check_guards): base pointer, user bytes, name.
   struct Guarded {
     char* base;
@@ -287,10 +292,11 @@ int check_guards(Batch* b) {
 }
 
 void drop_graphs(Batch* b) {
-  for (auto& g : b->graph)
-    if (g) {
-      cudaGraphExecDestroy(g);
-      g = nullptr;
+  for (int k = 0; k <= kGraphLog; ++k)
+    for (int c = 0; c < 2; ++c) {
+      if (b->graph[k][c]) cudaGraphExecDestroy(b->graph[k][c]);
+      b->graph[k][c] = nullptr;
+      b->graph_uses[k][c] = 0;
     }
 }
 
@@ -479,12 +485,23 @@ int default_rows(const Batch* b) {
   return r6;
 }
 
+// Whether steps of `items` CTAs on their own are launched as programmatic dependents, so that a
+// step's CTAs are resident and past their start-up when the step before ends: if two steps fit
+// on the GPU together (64 x 64: 3.1 us a step without, 2.5 with; 601 x 407: 6.7 and 6.0), or if
+// one fills it, so that each CTA that ends makes room for one (1024^2: 14.1 and 13.5).  In
+// between, the next step's first CTAs take the free places and the rest those of the SMs that
+// finish first, which ends up uneven (512^2 with 10 of 18 places taken: 6.5 and 9.0).
+bool overlap_ok(long long items, int occ, int sms) {
+  return 2 * items <= (long long)occ * sms || (items + sms - 1) / sms >= occ;
+}
+
 // CTA width and chunk height of a single lattice stepped with one launch per step, from a
 // model of the step's time: the time of a step alone on the GPU plus its work, the SM time of
 // all its CTAs, since lattices of a study often share the GPU.
 //
 // FP32 pair kernel, in us (fitted to 18 sizes from 64 x 64 to 1740 x 718, four widths and 14
-// heights, within 10 %): 2.4 for the launch and the first row, then per row (and one more of
+// heights, within 10 %): 2.4 for the launch and the first row (1.8 where steps overlap,
+// overlap_ok), then per row (and one more of
 // start-up) a latency and the issue of the W warps that the busiest SM holds; with more items
 // than resident CTAs, the work itself.  Chunks used to be eight rows at least: 64 x 64 stepped
 // in 7.4 us and takes 3.4 with one-row chunks, 601 x 407 in 9.6 and 6.9, and 1024^2 in 17.2
@@ -506,7 +523,8 @@ Tiling choose_pair_tiling(const Batch* b, const std::vector<int>& widths) {
       const long long k = (items + sms - 1) / sms;
       const double work = items * w * (rows + 1.5) * 0.0795 / sms;
       const double row = latency + 0.05 * std::min<long long>(k, occ) * w;
-      const double alone = 2.4 + (k <= occ ? (rows + 1) * row : work + 0.1 * (rows + 1) * row);
+      const double first = overlap_ok(items, occ, sms) ? 1.8 : 2.4;
+      const double alone = first + (k <= occ ? (rows + 1) * row : work + 0.1 * (rows + 1) * row);
       if (best_cost < 0 || alone + work < best_cost) {
         best_cost = alone + work;
         best = {nt, rows};
@@ -839,6 +857,8 @@ int rebuild_items(Batch* b) {
     int rc = build_persist(b);
     if (rc) return rc;
   }
+  b->dependent = !b->fp64 && b->vec == 2 && b->n_groups == 1 &&
+                 overlap_ok(b->n_items, lbm::pair_occupancy(b->rule, b->grp_nt[0]), b->sms);
   // Full-width strips neither read nor write the ghost columns, so after steps under one set
   // of work lists they may be stale; a pass under the new lists may use strips that read
   // them.
@@ -1003,8 +1023,9 @@ int create_batch(Batch* b, int n, const lbm_instance* in, bool fp64, int psi_fp6
   return rebuild_items(b);
 }
 
-// One step of the instances of launch group g, from slab c into slab c ^ 1.
-int launch_group(Batch* b, int g, int c, cudaStream_t st) {
+// One step of the instances of launch group g, from slab c into slab c ^ 1; dependent: as a
+// programmatic dependent of the stream's previous kernel, the group's previous step.
+int launch_group(Batch* b, int g, int c, bool dependent, cudaStream_t st) {
   const WorkItem* items = b->d_items + b->grp_begin[g];
   const int n = b->grp_begin[g + 1] - b->grp_begin[g];
   cudaError_t e;
@@ -1015,11 +1036,13 @@ int launch_group(Batch* b, int g, int c, cudaStream_t st) {
                                   st);
   } else if (b->vec == 2) {
     e = lbm::launch_pair(b->rule, b->grp_nt[g], b->grp_full[g], b->maps_step, c,
-                         (float*)b->slab[c ^ 1], b->d_inst, items, n, b->d_status, b->shared, st);
+                         (float*)b->slab[c ^ 1], b->d_inst, items, n, b->d_status, b->shared,
+                         dependent, st);
   } else {
     MomArgs<float> mo{};
     e = lbm::launch_sweep<float>(b->grp_nt[g], lbm::MODE_STEP, b->grp_full[g], (const float*)b->slab[c],
-                                 (float*)b->slab[c ^ 1], b->d_inst, items, n, mo, b->d_status, st);
+                                 (float*)b->slab[c ^ 1], b->d_inst, items, n, mo, b->d_status,
+                                 st);
   }
   if (e != cudaSuccess)
     return set_err(b->err, LBM_ECUDA, "step kernel launch failed: %s", cudaGetErrorString(e));
@@ -1038,16 +1061,6 @@ int launch_persist_steps(Batch* b, int c, int n, cudaStream_t st) {
                             b->persist_grid, lbm::DEP_WAIT_LIMIT, b->shared, st);
   if (e != cudaSuccess)
     return set_err(b->err, LBM_ECUDA, "persistent step launch failed: %s", cudaGetErrorString(e));
-  return LBM_OK;
-}
-
-// One step of every active instance: the launch groups one after another on st.
-int launch_step(Batch* b, cudaStream_t st) {
-  for (int g = 0; g < b->n_groups; ++g) {
-    int rc = launch_group(b, g, b->cur, st);
-    if (rc) return rc;
-  }
-  b->cur ^= 1;
   return LBM_OK;
 }
 
@@ -1071,8 +1084,8 @@ int queue_steps(Batch* b, int n, cudaStream_t st) {
   if (b->persist) return n > 0 ? launch_persist_steps(b, start, n, st) : LBM_OK;
   if (b->n_groups <= 1) {
     int rc = LBM_OK;
-    for (int k = 0; k < n && rc == LBM_OK; ++k) rc = launch_step(b, st);
-    b->cur = start;
+    for (int k = 0; k < n && b->n_groups == 1 && rc == LBM_OK; ++k)
+      rc = launch_group(b, 0, start ^ (k & 1), k > 0 && b->dependent, st);
     return rc;
   }
   int rc = ensure_branches(b);
@@ -1084,7 +1097,7 @@ int queue_steps(Batch* b, int n, cudaStream_t st) {
     return set_err(b->err, LBM_ECUDA, "stream fork failed: %s", cudaGetErrorString(e));
   for (int gi = 0; gi < b->n_groups && rc == LBM_OK; ++gi) {
     cudaStream_t sg = gi == 0 ? st : b->grp_stream[gi - 1];
-    for (int k = 0; k < n && rc == LBM_OK; ++k) rc = launch_group(b, gi, start ^ (k & 1), sg);
+    for (int k = 0; k < n && rc == LBM_OK; ++k) rc = launch_group(b, gi, start ^ (k & 1), false, sg);
   }
   // Join every branch that was forked, even after a failed launch.
   for (int k = 0; k + 1 < b->n_groups; ++k) {
@@ -1096,9 +1109,8 @@ int queue_steps(Batch* b, int n, cudaStream_t st) {
   return rc;
 }
 
-// Capture kGraphSteps consecutive steps that start from slab `start` (one branch per
-// launch group).
-int capture_graph(Batch* b, int start) {
+// Capture 2^k consecutive steps that start from slab `start` (one branch per launch group).
+int capture_graph(Batch* b, int k, int start) {
   const int saved = b->cur;
   if (b->n_groups > 1) {
     int rc = ensure_branches(b);  // created outside the capture
@@ -1107,7 +1119,7 @@ int capture_graph(Batch* b, int start) {
   b->cur = start;
   cudaGraph_t g = nullptr;
   CK(b, cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-  int rc = queue_steps(b, kGraphSteps, b->cap_stream);
+  int rc = queue_steps(b, 1 << k, b->cap_stream);
   cudaError_t e = cudaStreamEndCapture(b->cap_stream, &g);
   b->cur = saved;
   if (rc) {
@@ -1116,10 +1128,10 @@ int capture_graph(Batch* b, int start) {
   }
   if (e != cudaSuccess)
     return set_err(b->err, LBM_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
-  e = cudaGraphInstantiate(&b->graph[start], g, 0);
+  e = cudaGraphInstantiate(&b->graph[k][start], g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) {
-    b->graph[start] = nullptr;
+    b->graph[k][start] = nullptr;
     return set_err(b->err, LBM_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
   }
   return LBM_OK;
@@ -1129,19 +1141,28 @@ int do_steps(Batch* b, long long n) {
   if (n < 0) return set_err(b->err, LBM_EINVAL, "step count must be >= 0");
   if (b->n_items == 0) return LBM_OK;
   const long long n0 = n;
+  // Runs of kGraphSteps are replayed from a graph, and so are the powers of two of what is
+  // left, once a run of that length comes back (36 launches of a 100-step call kept the host
+  // busy for 80 us, more than the steps of a small lattice take); a persistent run of any
+  // length is one launch.
   while (n > 0) {
-    if (n >= kGraphSteps) {
-      if (!b->graph[b->cur]) {
-        int rc = capture_graph(b, b->cur);
+    int k = kGraphLog;
+    while (k > 0 && (1LL << k) > n) --k;
+    const bool whole = k == kGraphLog;
+    if (whole || (k > 0 && !b->persist && b->graph_uses[k][b->cur] > 0)) {
+      if (!b->graph[k][b->cur]) {
+        int rc = capture_graph(b, k, b->cur);
         if (rc) return rc;
       }
-      CK(b, cudaGraphLaunch(b->graph[b->cur], b->stream));
-      n -= kGraphSteps;
+      CK(b, cudaGraphLaunch(b->graph[k][b->cur], b->stream));
+      n -= 1LL << k;
     } else {
-      int rc = queue_steps(b, (int)n, b->stream);
+      const int m = b->persist ? (int)n : 1 << k;
+      int rc = queue_steps(b, m, b->stream);
       if (rc) return rc;
-      b->cur ^= (int)(n & 1);
-      n = 0;
+      ++b->graph_uses[k][b->cur];
+      b->cur ^= m & 1;
+      n -= m;
     }
   }
   for (int i = 0; i < b->n_inst; ++i)

@@ -18,16 +18,20 @@ cudaError_t launch_sweep(int nt, int mode, int full, const S* fin, S* fout, cons
 // kind (full-width strips or not; a CTA whose instance is of the other kind returns at
 // once), and a step for a viscosity rule (VISC_* with the constants that the instances of the
 // launch share, or PAIR_ANY).  Both read the slab of the given index through the row maps.
+// dependent: launched as a programmatic dependent of the stream's previous kernel, which must
+// be the previous step.
 cudaError_t launch_pair_moments(int nt, int full, const RowMaps& maps, int slab,
                                 const InstParams* d_inst, const WorkItem* d_items, int n_items,
                                 const MomArgs<float>& mo, int* d_status, cudaStream_t st);
 cudaError_t launch_pair(int rule, int nt, int full, const RowMaps& maps, int slab, float* fout,
                         const InstParams* d_inst, const WorkItem* d_items, int n_items,
-                        int* d_status, const PairConsts& shared, cudaStream_t st);
+                        int* d_status, const PairConsts& shared, bool dependent,
+                        cudaStream_t st);
 template <int RULE>
 cudaError_t launch_pair_step(int nt, int full, const RowMaps& maps, int slab, float* fout,
                              const InstParams* d_inst, const WorkItem* d_items, int n_items,
-                             int* d_status, const PairConsts& shared, cudaStream_t st);
+                             int* d_status, const PairConsts& shared, bool dependent,
+                             cudaStream_t st);
 template <int RULE>
 cudaError_t launch_pair_persist(int nt, int kind, const RowMaps& maps, int slab,
                                 float* slab0, float* slab1,

@@ -20,9 +20,9 @@ cudaError_t launch_pair_moments(int nt, int full, const RowMaps& maps, int slab,
 #define LBM_PAIR_MOM(T)                                                                     \
   if (nt == T)                                                                              \
     return full ? launch_sweep2_cfg<T, MODE_MOMENTS, true, PAIR_ANY>(                       \
-                      maps, slab, nullptr, d_inst, d_items, n_items, mo, d_status, none, st) \
+                      maps, slab, nullptr, d_inst, d_items, n_items, mo, d_status, none, false, st) \
                 : launch_sweep2_cfg<T, MODE_MOMENTS, false, PAIR_ANY>(                      \
-                      maps, slab, nullptr, d_inst, d_items, n_items, mo, d_status, none, st);
+                      maps, slab, nullptr, d_inst, d_items, n_items, mo, d_status, none, false, st);
   LBM_PAIR_MOM(32)
   LBM_PAIR_MOM(64)
   LBM_PAIR_MOM(96)

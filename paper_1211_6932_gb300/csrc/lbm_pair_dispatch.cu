@@ -14,9 +14,10 @@ namespace lbm {
 
 cudaError_t launch_pair(int rule, int nt, int full, const RowMaps& maps, int slab, float* fout,
                         const InstParams* d_inst, const WorkItem* d_items, int n_items,
-                        int* d_status, const PairConsts& shared, cudaStream_t st) {
+                        int* d_status, const PairConsts& shared, bool dependent,
+                        cudaStream_t st) {
   LBM_BY_RULE(launch_pair_step, nt, full, maps, slab, fout, d_inst, d_items, n_items, d_status, shared,
-              st)
+              dependent, st)
 }
 
 cudaError_t launch_persist(int rule, int nt, int kind, const RowMaps& maps, int slab,

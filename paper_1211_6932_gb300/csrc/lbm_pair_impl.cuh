@@ -5,19 +5,36 @@
 
 namespace lbm {
 
+// Launch a kernel, as a programmatic dependent of the stream's previous kernel if asked
+// (step_begin waits for that one's completion).
+template <typename... P, typename... A>
+static cudaError_t launch_kernel(void (*kernel)(P...), int blocks, int threads, size_t smem,
+                                 bool dependent, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <int NT, int MODE, bool FULL, int VISC>
 static cudaError_t launch_sweep2_cfg(const RowMaps& maps, int slab, float* fout, const InstParams* d_inst,
                                      const WorkItem* d_items, int n_items,
                                      const MomArgs<float>& mo, int* d_status,
-                                     const PairConsts& shared, cudaStream_t st) {
+                                     const PairConsts& shared, bool dependent, cudaStream_t st) {
   constexpr size_t smem = Sweep2Cfg<NT>::BYTES;
   static std::atomic<unsigned long long> done{0};
   cudaError_t e = ensure_smem_attr(sweep2_kernel<NT, MODE, FULL, VISC>, smem, done);
   if (e != cudaSuccess) return e;
   if (n_items <= 0) return cudaSuccess;
-  sweep2_kernel<NT, MODE, FULL, VISC><<<n_items, NT, smem, st>>>(
-      maps, slab, fout, d_inst, d_items, n_items, mo, d_status, shared);
-  return cudaGetLastError();
+  return launch_kernel(sweep2_kernel<NT, MODE, FULL, VISC>, n_items, NT, smem, dependent, st, maps,
+                       slab, fout, d_inst, d_items, n_items, mo, d_status, shared);
 }
 
 // Persistent pair kernel (sweep2_persist_kernel) with `grid` CTAs.
@@ -49,16 +66,17 @@ static int pair_occupancy(F* fn, int nt, size_t smem) {
 template <int VISC>
 cudaError_t launch_pair_step(int nt, int full, const RowMaps& maps, int slab, float* fout,
                              const InstParams* d_inst, const WorkItem* d_items, int n_items,
-                             int* d_status, const PairConsts& shared, cudaStream_t st) {
+                             int* d_status, const PairConsts& shared, bool dependent,
+                             cudaStream_t st) {
   const MomArgs<float> mo{};
 #define LBM_PAIR(T)                                                                           \
   if (nt == T)                                                                                \
     return full ? launch_sweep2_cfg<T, MODE_STEP, true, VISC>(maps, slab, fout, d_inst, d_items,     \
                                                               n_items, mo, d_status, shared,  \
-                                                              st)                             \
+                                                              dependent, st)                             \
                 : launch_sweep2_cfg<T, MODE_STEP, false, VISC>(maps, slab, fout, d_inst, d_items,    \
                                                                n_items, mo, d_status, shared, \
-                                                               st);
+                                                               dependent, st);
   LBM_PAIR(32)
   LBM_PAIR(64)
   LBM_PAIR(96)
@@ -129,7 +147,7 @@ int pair_step_occupancy(int nt) {
 #define LBM_INSTANTIATE_PAIR(V)                                                               \
   template cudaError_t lbm::launch_pair_step<V>(int, int, const lbm::RowMaps&, int, float*,               \
                                                 const lbm::InstParams*, const lbm::WorkItem*, \
-                                                int, int*, const lbm::PairConsts&,            \
+                                                int, int*, const lbm::PairConsts&, bool,      \
                                                 cudaStream_t);                                \
   template cudaError_t lbm::launch_pair_persist<V>(                                           \
       int, int, const lbm::RowMaps&, int, float*, float*, const lbm::InstParams*,          \
