@@ -1145,11 +1145,15 @@ int do_steps(Batch* b, long long n) {
   // left, once a run of that length comes back (36 launches of a 100-step call kept the host
   // busy for 80 us, more than the steps of a small lattice take); a persistent run of any
   // length is one launch.
+  // A caller's own capture of a short run gets its launches, as it did.
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(b->stream, &capture) != cudaSuccess) cudaGetLastError();
+  const bool replay = !b->persist && capture == cudaStreamCaptureStatusNone;
   while (n > 0) {
     int k = kGraphLog;
     while (k > 0 && (1LL << k) > n) --k;
     const bool whole = k == kGraphLog;
-    if (whole || (k > 0 && !b->persist && b->graph_uses[k][b->cur] > 0)) {
+    if (whole || (k > 0 && replay && b->graph_uses[k][b->cur] > 0)) {
       if (!b->graph[k][b->cur]) {
         int rc = capture_graph(b, k, b->cur);
         if (rc) return rc;
