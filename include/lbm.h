@@ -89,7 +89,9 @@ typedef struct {
   void* stream;   /* cudaStream_t to queue work on; NULL: a stream the handle owns */
   int device;     /* CUDA device ordinal; -1 (default): the library's current device.
                      Every call on the handle makes this device current first. */
-  int tile_threads; /* threads per CTA of the step kernel; 0 (default): 128.
+  int tile_threads; /* threads per CTA of the step kernel; 0 (default): 128, or, for a single
+                       lattice at the default tile_vec and tile_rows 0 that does not step
+                       persistently, chosen with the chunk height (tile_rows).
                        LBM_TILE_PER_INSTANCE (FP32_DEV with tile_vec 2 only): each
                        instance gets the pair-kernel width (32, 64, 96 or 128 threads)
                        that wastes least of its columns; one launch per width and kind of
@@ -97,11 +99,12 @@ typedef struct {
   int tile_vec;     /* adjacent columns per thread: 1, or 2 (FP32 only: packed float2
                        arithmetic); available (threads, vec) pairs: FP32 (64|128|256, 1),
                        (32|64|96|128, 2); FP64 (64|128, 1).  0 (default): 2 for FP32_DEV,
-                       1 for FP64.  A CTA owns threads*vec - 4 columns; with vec 2 a
-                       lattice of at most 2*threads columns is swept in one full-width
+                       1 for FP64.  A CTA owns threads*vec - 4 columns; a
+                       lattice of at most threads*vec columns is swept in one full-width
                        strip per row (all threads own columns, x wraps in shared memory,
                        no ghost columns read or written). */
-  int tile_rows;  /* rows per CTA sweep; 0 (default): sized to fill the GPU */
+  int tile_rows;  /* rows per CTA sweep; 0 (default): sized to fill the GPU (for a single
+                     lattice by a model of the step's time, down to one row) */
 } lbm_options;
 
 typedef struct lbm_handle lbm_handle;
@@ -177,8 +180,8 @@ int lbm_get_populations(lbm_handle* h, double* f);
 /*
  * Advance n >= 0 time steps (Eqs. 1-7 with the forcing of Eq. 25, Sec. II-III).  Each
  * step is one pass of the fused kernel: one launch per step, or, stepping persistently
- * (see lbm_persistent), one launch per run of up to 64 steps; runs of 64 steps are
- * replayed from a CUDA graph.
+ * (see lbm_persistent), one launch per run of up to 64 steps; runs of 64 steps, and the
+ * powers of two below once they come back, are replayed from a CUDA graph.
  * Asynchronous: returns once the work is queued.  Status is reported by lbm_sync and by
  * every synchronous call.
  */

@@ -465,7 +465,7 @@ int default_rows(const Batch* b) {
     if (b->active[i]) {
       const int nt = step_nt(b, i);
       const int occ = b->fp64 ? lbm::sweep_occupancy<double>(nt)
-                      : b->vec == 2 ? lbm::pair_occupancy(b->rule, nt)
+                      : b->vec == 2 ? lbm::pair_occupancy(b->rule, nt, 8)
                                     : lbm::sweep_occupancy<float>(nt);
       sm_rows += (double)lbm::strips_for(b->inst[i].nx, nt, b->vec) * b->inst[i].ny /
                  std::max(occ, 1);
@@ -487,7 +487,7 @@ int default_rows(const Batch* b) {
 
 // Whether steps of `items` CTAs on their own are launched as programmatic dependents, so that a
 // step's CTAs are resident and past their start-up when the step before ends: if two steps fit
-// on the GPU together (64 x 64: 3.1 us a step without, 2.5 with; 601 x 407: 6.7 and 6.0), or if
+// on the GPU together (64 x 64: 3.1 us a step without, 2.6 with; 601 x 407: 6.7 and 6.0), or if
 // one fills it, so that each CTA that ends makes room for one (1024^2: 14.1 and 13.5).  In
 // between, the next step's first CTAs take the free places and the rest those of the SMs that
 // finish first, which ends up uneven (512^2 with 10 of 18 places taken: 6.5 and 9.0).
@@ -504,8 +504,8 @@ bool overlap_ok(long long items, int occ, int sms) {
 // overlap_ok), then per row (and one more of
 // start-up) a latency and the issue of the W warps that the busiest SM holds; with more items
 // than resident CTAs, the work itself.  Chunks used to be eight rows at least: 64 x 64 stepped
-// in 7.4 us and takes 3.4 with one-row chunks, 601 x 407 in 9.6 and 6.9, and 1024^2 in 17.2
-// (strips of 252 columns cover 1260) and 14.7 (six of 188 cover 1128).
+// in 7.4 us and takes 2.3 with one-row chunks, 601 x 407 in 9.6 and 6.0, and 1024^2 in 17.2
+// (strips of 252 columns cover 1260) and 13.5 (six of 188 cover 1128).
 struct Tiling {
   int nt, rows;
 };
@@ -515,10 +515,12 @@ Tiling choose_pair_tiling(const Batch* b, const std::vector<int>& widths) {
   Tiling best{widths[0], 8};
   double best_cost = -1.0;
   for (int nt : widths) {
-    const int occ = lbm::pair_occupancy(b->rule, nt);
+    const int occ3[3] = {lbm::pair_occupancy(b->rule, nt, 1), lbm::pair_occupancy(b->rule, nt, 2),
+                         lbm::pair_occupancy(b->rule, nt, 3)};
     const long long strips = lbm::strips_for(P.nx, nt, 2);
     const double w = nt / 32.0, latency = lbm::full_width(P.nx, nt, 2) ? 0.40 : 0.62;
     for (int rows = 1; rows <= 64; ++rows) {
+      const int occ = occ3[std::min(rows, 3) - 1];
       const long long items = strips * ((P.ny + rows - 1) / rows);
       const long long k = (items + sms - 1) / sms;
       const double work = items * w * (rows + 1.5) * 0.0795 / sms;
@@ -858,7 +860,7 @@ int rebuild_items(Batch* b) {
     if (rc) return rc;
   }
   b->dependent = !b->fp64 && b->vec == 2 && b->n_groups == 1 &&
-                 overlap_ok(b->n_items, lbm::pair_occupancy(b->rule, b->grp_nt[0]), b->sms);
+                 overlap_ok(b->n_items, lbm::pair_occupancy(b->rule, b->grp_nt[0], b->rows), b->sms);
   // Full-width strips neither read nor write the ghost columns, so after steps under one set
   // of work lists they may be stale; a pass under the new lists may use strips that read
   // them.
@@ -1035,7 +1037,7 @@ int launch_group(Batch* b, int g, int c, bool dependent, cudaStream_t st) {
                                   (double*)b->slab[c ^ 1], b->d_inst, items, n, mo, b->d_status,
                                   st);
   } else if (b->vec == 2) {
-    e = lbm::launch_pair(b->rule, b->grp_nt[g], b->grp_full[g], b->maps_step, c,
+    e = lbm::launch_pair(b->rule, b->grp_nt[g], b->rows, b->grp_full[g], b->maps_step, c,
                          (float*)b->slab[c ^ 1], b->d_inst, items, n, b->d_status, b->shared,
                          dependent, st);
   } else {

@@ -18,17 +18,20 @@ cudaError_t launch_sweep(int nt, int mode, int full, const S* fin, S* fout, cons
 // kind (full-width strips or not; a CTA whose instance is of the other kind returns at
 // once), and a step for a viscosity rule (VISC_* with the constants that the instances of the
 // launch share, or PAIR_ANY).  Both read the slab of the given index through the row maps.
-// dependent: launched as a programmatic dependent of the stream's previous kernel, which must
-// be the previous step.
+// rows: the items' chunk height (one and two rows have a kernel of their own); dependent:
+// launched as a programmatic dependent of the stream's previous kernel, which must be the
+// previous step.
 cudaError_t launch_pair_moments(int nt, int full, const RowMaps& maps, int slab,
                                 const InstParams* d_inst, const WorkItem* d_items, int n_items,
                                 const MomArgs<float>& mo, int* d_status, cudaStream_t st);
-cudaError_t launch_pair(int rule, int nt, int full, const RowMaps& maps, int slab, float* fout,
+cudaError_t launch_pair(int rule, int nt, int rows, int full, const RowMaps& maps, int slab,
+                        float* fout,
                         const InstParams* d_inst, const WorkItem* d_items, int n_items,
                         int* d_status, const PairConsts& shared, bool dependent,
                         cudaStream_t st);
 template <int RULE>
-cudaError_t launch_pair_step(int nt, int full, const RowMaps& maps, int slab, float* fout,
+cudaError_t launch_pair_step(int nt, int rows, int full, const RowMaps& maps, int slab,
+                             float* fout,
                              const InstParams* d_inst, const WorkItem* d_items, int n_items,
                              int* d_status, const PairConsts& shared, bool dependent,
                              cudaStream_t st);
@@ -42,9 +45,9 @@ cudaError_t launch_pair_persist(int nt, int kind, const RowMaps& maps, int slab,
 template <int RULE>
 int pair_persist_occupancy(int nt, int kind);
 template <int RULE>
-int pair_step_occupancy(int nt);
-// Resident CTAs per SM of the pair kernel's step (at least 1).
-int pair_occupancy(int rule, int nt);
+int pair_step_occupancy(int nt, int rows);
+// Resident CTAs per SM of the pair kernel's step for chunks of `rows` rows (at least 1).
+int pair_occupancy(int rule, int nt, int rows);
 template <typename S>
 cudaError_t launch_fill_ghosts(S* buf, const InstParams& P, cudaStream_t st);
 template <typename S>

@@ -12,11 +12,12 @@ namespace lbm {
     default: return FN<PAIR_ANY>(__VA_ARGS__);                                     \
   }
 
-cudaError_t launch_pair(int rule, int nt, int full, const RowMaps& maps, int slab, float* fout,
+cudaError_t launch_pair(int rule, int nt, int rows, int full, const RowMaps& maps, int slab,
+                        float* fout,
                         const InstParams* d_inst, const WorkItem* d_items, int n_items,
                         int* d_status, const PairConsts& shared, bool dependent,
                         cudaStream_t st) {
-  LBM_BY_RULE(launch_pair_step, nt, full, maps, slab, fout, d_inst, d_items, n_items, d_status, shared,
+  LBM_BY_RULE(launch_pair_step, nt, rows, full, maps, slab, fout, d_inst, d_items, n_items, d_status, shared,
               dependent, st)
 }
 
@@ -34,6 +35,6 @@ int persist_occupancy(int rule, int nt, int kind) {
   LBM_BY_RULE(pair_persist_occupancy, nt, kind)
 }
 
-int pair_occupancy(int rule, int nt) { LBM_BY_RULE(pair_step_occupancy, nt) }
+int pair_occupancy(int rule, int nt, int rows) { LBM_BY_RULE(pair_step_occupancy, nt, rows) }
 
 }  // namespace lbm

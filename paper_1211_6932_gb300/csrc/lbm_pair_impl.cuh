@@ -37,6 +37,21 @@ static cudaError_t launch_sweep2_cfg(const RowMaps& maps, int slab, float* fout,
                        slab, fout, d_inst, d_items, n_items, mo, d_status, shared);
 }
 
+// Chunks of at most ROWS rows (sweep2_short_kernel).
+template <int NT, int ROWS, bool FULL, int VISC>
+static cudaError_t launch_short_cfg(const RowMaps& maps, int slab, float* fout,
+                                    const InstParams* d_inst, const WorkItem* d_items,
+                                    int n_items, int* d_status, const PairConsts& shared,
+                                    bool dependent, cudaStream_t st) {
+  constexpr size_t smem = ShortCfg<NT, ROWS>::BYTES;
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = ensure_smem_attr(sweep2_short_kernel<NT, ROWS, FULL, VISC>, smem, done);
+  if (e != cudaSuccess) return e;
+  if (n_items <= 0) return cudaSuccess;
+  return launch_kernel(sweep2_short_kernel<NT, ROWS, FULL, VISC>, n_items, NT, smem, dependent, st,
+                       maps, slab, fout, d_inst, d_items, n_items, d_status, shared);
+}
+
 // Persistent pair kernel (sweep2_persist_kernel) with `grid` CTAs.
 template <int NT, int KIND, int VISC>
 static cudaError_t launch_persist2_cfg(const RowMaps& maps, int slab, float* slab0, float* slab1, const InstParams* d_inst,
@@ -64,24 +79,30 @@ static int pair_occupancy(F* fn, int nt, size_t smem) {
 }
 
 template <int VISC>
-cudaError_t launch_pair_step(int nt, int full, const RowMaps& maps, int slab, float* fout,
-                             const InstParams* d_inst, const WorkItem* d_items, int n_items,
-                             int* d_status, const PairConsts& shared, bool dependent,
-                             cudaStream_t st) {
+cudaError_t launch_pair_step(int nt, int rows, int full, const RowMaps& maps, int slab,
+                             float* fout, const InstParams* d_inst, const WorkItem* d_items,
+                             int n_items, int* d_status, const PairConsts& shared,
+                             bool dependent, cudaStream_t st) {
   const MomArgs<float> mo{};
-#define LBM_PAIR(T)                                                                           \
-  if (nt == T)                                                                                \
-    return full ? launch_sweep2_cfg<T, MODE_STEP, true, VISC>(maps, slab, fout, d_inst, d_items,     \
-                                                              n_items, mo, d_status, shared,  \
-                                                              dependent, st)                             \
-                : launch_sweep2_cfg<T, MODE_STEP, false, VISC>(maps, slab, fout, d_inst, d_items,    \
-                                                               n_items, mo, d_status, shared, \
-                                                               dependent, st);
+#define LBM_PAIR_KIND(T, F)                                                                    \
+  if (nt == T && (full != 0) == F)                                                             \
+    return rows == 1   ? launch_short_cfg<T, 1, F, VISC>(maps, slab, fout, d_inst, d_items,    \
+                                                         n_items, d_status, shared, dependent, \
+                                                         st)                                   \
+           : rows == 2 ? launch_short_cfg<T, 2, F, VISC>(maps, slab, fout, d_inst, d_items,    \
+                                                         n_items, d_status, shared, dependent, \
+                                                         st)                                   \
+                       : launch_sweep2_cfg<T, MODE_STEP, F, VISC>(maps, slab, fout, d_inst,    \
+                                                                  d_items, n_items, mo,        \
+                                                                  d_status, shared, dependent, \
+                                                                  st);
+#define LBM_PAIR(T) LBM_PAIR_KIND(T, true) LBM_PAIR_KIND(T, false)
   LBM_PAIR(32)
   LBM_PAIR(64)
   LBM_PAIR(96)
   LBM_PAIR(128)
 #undef LBM_PAIR
+#undef LBM_PAIR_KIND
   return cudaErrorInvalidValue;
 }
 
@@ -130,10 +151,15 @@ int pair_persist_occupancy(int nt, int kind) {
 }
 
 template <int VISC>
-int pair_step_occupancy(int nt) {
-#define LBM_PAIR_OCC(T)                                                              \
-  if (nt == T)                                                                       \
-    return pair_occupancy(sweep2_kernel<T, MODE_STEP, false, VISC>, T, Sweep2Cfg<T>::BYTES);
+int pair_step_occupancy(int nt, int rows) {
+#define LBM_PAIR_OCC(T)                                                                       \
+  if (nt == T)                                                                                \
+    return rows == 1   ? pair_occupancy(sweep2_short_kernel<T, 1, false, VISC>, T,            \
+                                        ShortCfg<T, 1>::BYTES)                                \
+           : rows == 2 ? pair_occupancy(sweep2_short_kernel<T, 2, false, VISC>, T,            \
+                                        ShortCfg<T, 2>::BYTES)                                \
+                       : pair_occupancy(sweep2_kernel<T, MODE_STEP, false, VISC>, T,          \
+                                        Sweep2Cfg<T>::BYTES);
   LBM_PAIR_OCC(32)
   LBM_PAIR_OCC(64)
   LBM_PAIR_OCC(96)
@@ -145,7 +171,7 @@ int pair_step_occupancy(int nt) {
 }  // namespace lbm
 
 #define LBM_INSTANTIATE_PAIR(V)                                                               \
-  template cudaError_t lbm::launch_pair_step<V>(int, int, const lbm::RowMaps&, int, float*,               \
+  template cudaError_t lbm::launch_pair_step<V>(int, int, int, const lbm::RowMaps&, int, float*,               \
                                                 const lbm::InstParams*, const lbm::WorkItem*, \
                                                 int, int*, const lbm::PairConsts&, bool,      \
                                                 cudaStream_t);                                \
@@ -155,4 +181,4 @@ int pair_step_occupancy(int nt) {
       const lbm::ItemLink*, int, int, int*, int*, int*, int, int, const lbm::PairConsts&,     \
       cudaStream_t);                                                                          \
   template int lbm::pair_persist_occupancy<V>(int, int);                                      \
-  template int lbm::pair_step_occupancy<V>(int);
+  template int lbm::pair_step_occupancy<V>(int, int);

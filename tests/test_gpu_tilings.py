@@ -1,6 +1,6 @@
 """Every tiling of the pair kernel gives the same bits (the arithmetic of a node does not
 depend on the CTA that computes it), so the default tiling of small and ragged lattices,
-with chunks down to one row, is compared with chunks of eight rows of 128-thread CTAs: full
+with chunks down to one row (one and two rows have a kernel of their own), is compared with chunks of eight rows of 128-thread CTAs: full
 width and strips, even and odd widths (ghost columns written as pairs and one by one), a last
 strip of one column or of two, walls."""
 import numpy as np
@@ -22,7 +22,7 @@ def test_default_tiling_equals_eight_row_chunks(walls):
         f = pairs.droplet_state(c, vel=0.02, seed=k)
         got = []
         for kw in ({}, {"tile_threads": 128, "tile_rows": 8}, {"tile_threads": 32, "tile_rows": 1},
-                   {"tile_threads": 64, "tile_rows": 3}):
+                   {"tile_threads": 96, "tile_rows": 2}, {"tile_threads": 64, "tile_rows": 3}):
             with pairs.gpu_lattice(c, "fp32", **kw) as L:
                 L.set_populations(f)
                 L.step(70)
