@@ -538,7 +538,7 @@ Tiling choose_pair_tiling(const Batch* b, const std::vector<int>& widths) {
 
 // FP64, whose kernel is bound by the FP64 pipe: a row of a 64-thread CTA keeps an SM's pipe
 // for 2.4 us (and takes 5.2 alone), a chunk costs its rows and 0.73 of one for the psi of its
-// halo rows.  128^2 runs in 11.5 us a step with one full-width CTA of 128 a row (14.9 with
+// halo rows.  128^2 runs in 9.3 us a step with one full-width CTA of 128 a row (13.5 with
 // strips of 60), 500 x 400 in 68 with 64 x 6 (116 with 128 x 4).
 Tiling choose_fp64_tiling(const Batch* b, const std::vector<int>& widths) {
   const InstParams& P = b->inst[0];
@@ -766,35 +766,36 @@ TensorMapEncodeFn tensor_map_encoder() {
 }
 
 // Tensor map of instance P's rows in a slab for CTAs of nt threads: elements are pairs of
-// floats (a box may have 256 elements a side, a 128-thread row has 260 floats), and rows are
-// copied from a column that is a multiple of four floats, so every copy starts on 16 bytes.
-int row_map(Batch* b, const InstParams& P, float* slab, int nt, CUtensorMap* map) {
+// floats (a box may have 256 elements a side, a 128-thread row has 260 floats) or doubles,
+// and rows are copied from a column that is a multiple of four, so every copy starts on 16
+// bytes.
+int row_map(Batch* b, const InstParams& P, void* slab, int nt, CUtensorMap* map) {
   TensorMapEncodeFn encode = tensor_map_encoder();
   if (!encode) return set_err(b->err, LBM_ECUDA, "cuTensorMapEncodeTiled is not available");
-  const cuuint64_t dim[3] = {(cuuint64_t)P.pitch / 2, (cuuint64_t)P.ny, (cuuint64_t)lbm::Q};
-  const cuuint64_t stride[2] = {(cuuint64_t)P.pitch * sizeof(float),
-                                (cuuint64_t)P.plane * sizeof(float)};
-  const cuuint32_t box[3] = {(cuuint32_t)(2 * nt + 4) / 2, 1, (cuuint32_t)lbm::Q};
+  const int per = b->fp64 ? 1 : 2;  // values an element
+  const cuuint64_t dim[3] = {(cuuint64_t)(P.pitch / per), (cuuint64_t)P.ny, (cuuint64_t)lbm::Q};
+  const cuuint64_t stride[2] = {(cuuint64_t)P.pitch * b->esz, (cuuint64_t)P.plane * b->esz};
+  const cuuint32_t box[3] = {(cuuint32_t)(nt * b->vec + 4) / per, 1, (cuuint32_t)lbm::Q};
   const cuuint32_t one[3] = {1, 1, 1};
   const CUresult r =
-      encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, slab + P.off, dim, stride, box, one,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+      encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, (char*)slab + P.off * b->esz, dim, stride,
+             box, one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS)
     return set_err(b->err, LBM_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
   return LBM_OK;
 }
 
-// Tensor maps for the current widths (pair tilings only).
+// Tensor maps for the current widths (pair tilings and FP64).
 int build_maps(Batch* b) {
-  if (b->fp64 || b->vec != 2) return LBM_OK;
+  if (!b->fp64 && b->vec != 2) return LBM_OK;
   const int n = b->n_inst;
   std::vector<CUtensorMap> maps(4 * (size_t)n);  // step maps (2 i + slab), then moments maps
   for (int i = 0; i < n; ++i)
     for (int k = 0; k < 2; ++k) {
-      int rc = row_map(b, b->inst[i], (float*)b->slab[k], step_nt(b, i), &maps[2 * i + k]);
+      int rc = row_map(b, b->inst[i], b->slab[k], step_nt(b, i), &maps[2 * i + k]);
       if (rc == LBM_OK)
-        rc = row_map(b, b->inst[i], (float*)b->slab[k], mom_nt(b), &maps[2 * (n + i) + k]);
+        rc = row_map(b, b->inst[i], b->slab[k], mom_nt(b), &maps[2 * (n + i) + k]);
       if (rc) return rc;
     }
   for (int k = 0; k < 2; ++k) {
@@ -1031,7 +1032,10 @@ int launch_group(Batch* b, int g, int c, bool dependent, cudaStream_t st) {
   const WorkItem* items = b->d_items + b->grp_begin[g];
   const int n = b->grp_begin[g + 1] - b->grp_begin[g];
   cudaError_t e;
-  if (b->fp64) {
+  if (b->fp64 && b->rows == 1) {
+    e = lbm::launch_short64(b->grp_nt[g], b->grp_full[g], b->maps_step, c,
+                            (double*)b->slab[c ^ 1], b->d_inst, items, n, b->d_status, st);
+  } else if (b->fp64) {
     MomArgs<double> mo{};
     e = lbm::launch_sweep<double>(b->grp_nt[g], lbm::MODE_STEP, b->grp_full[g], (const double*)b->slab[c],
                                   (double*)b->slab[c ^ 1], b->d_inst, items, n, mo, b->d_status,

@@ -14,6 +14,10 @@ template <typename S>
 cudaError_t launch_sweep(int nt, int mode, int full, const S* fin, S* fout, const InstParams* d_inst,
                          const WorkItem* d_items, int n_items, const MomArgs<S>& mo,
                          int* d_status, cudaStream_t st);
+// Step of FP64 items of one row each (short64_kernel), reading the given slab by row map.
+cudaError_t launch_short64(int nt, int full, const RowMaps& maps, int slab, double* fout,
+                           const InstParams* d_inst, const WorkItem* d_items, int n_items,
+                           int* d_status, cudaStream_t st);
 // Pair kernel (two columns per thread): the moments/diagnostics pass over the items of one
 // kind (full-width strips or not; a CTA whose instance is of the other kind returns at
 // once), and a step for a viscosity rule (VISC_* with the constants that the instances of the

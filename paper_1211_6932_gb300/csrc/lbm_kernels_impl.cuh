@@ -22,6 +22,24 @@ static cudaError_t ensure_smem_attr(F* fn, size_t smem, std::atomic<unsigned lon
   return e;
 }
 
+// Launch a kernel, as a programmatic dependent of the stream's previous kernel if asked
+// (step_begin waits for that one's completion).
+template <typename... P, typename... A>
+static cudaError_t launch_kernel(void (*kernel)(P...), int blocks, int threads, size_t smem,
+                                 bool dependent, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <typename S, int NT, int MODE, bool FULL>
 static cudaError_t launch_sweep_cfg(const S* fin, S* fout, const InstParams* d_inst,
                                     const WorkItem* d_items, int n_items, const MomArgs<S>& mo,

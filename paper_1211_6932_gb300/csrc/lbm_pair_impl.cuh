@@ -5,24 +5,6 @@
 
 namespace lbm {
 
-// Launch a kernel, as a programmatic dependent of the stream's previous kernel if asked
-// (step_begin waits for that one's completion).
-template <typename... P, typename... A>
-static cudaError_t launch_kernel(void (*kernel)(P...), int blocks, int threads, size_t smem,
-                                 bool dependent, cudaStream_t st, const A&... args) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)blocks);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = &at;
-  cfg.numAttrs = dependent ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
-}
-
 template <int NT, int MODE, bool FULL, int VISC>
 static cudaError_t launch_sweep2_cfg(const RowMaps& maps, int slab, float* fout, const InstParams* d_inst,
                                      const WorkItem* d_items, int n_items,
