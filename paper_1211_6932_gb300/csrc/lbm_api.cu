@@ -1861,48 +1861,55 @@ int autotune(Batch* b, int steps, const char* cache_path, TileChoice& best) {
   // Heights below 8 are for small grids, where more (shorter) chunks fill more SMs.
   const int rows_c[] = {1, 2, 4, 8, 12, 16, 20, 24, 28, 32, 40, 48, 64};
   best = TileChoice();
-  for (int vec : vecs) {
-    for (int nt : nts) {
-      if (!tiling_ok(b->fp64, nt, vec)) continue;
-      for (int rows : rows_c) {
-        // A tiling that steps persistently is timed that way and with one launch per step.
-        for (int persist = 1; persist >= 0 && rc == LBM_OK; --persist) {
-          rc = apply_tiling(b, nt, vec, rows, persist != 0);
-          if (rc) break;
-          const bool persistent = b->persist;
-          // Timed as stepping runs (graph replays for each kGraphSteps); an even count
-          // returns to the same slab, so the warm-up run captures the graph the timed run
-          // replays.
-          const int n_t = steps + (steps & 1);
-          rc = do_steps(b, n_t);  // warm-up
-          if (rc) break;
-          double per = -1.0;  // the better of two timed runs
-          for (int rep = 0; rep < 2; ++rep) {
-            if (!cu(cudaEventRecord(e0, b->stream), "cudaEventRecord")) break;
-            rc = do_steps(b, n_t);
-            if (rc) break;
-            if (!cu(cudaEventRecord(e1, b->stream), "cudaEventRecord")) break;
-            if (!cu(cudaEventSynchronize(e1), "cudaEventSynchronize")) break;
-            float ms = 0.f;
-            if (!cu(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime")) break;
-            if (per < 0 || ms / n_t < per) per = ms / n_t;
-          }
-          if (rc) break;
-          if (best.ms < 0 || per < best.ms) {
-            best.nt = nt;
-            best.vec = vec;
-            best.rows = rows;
-            best.ms = per;
-            best.persist = persist;
-          }
-          if (!persistent) break;  // the tiling does not step persistently: timed once
-        }
+  // A tiling that steps persistently is timed that way and with one launch per step.
+  auto time_tiling = [&](int nt, int vec, int rows) {
+    for (int persist = 1; persist >= 0 && rc == LBM_OK; --persist) {
+      rc = apply_tiling(b, nt, vec, rows, persist != 0);
+      if (rc) break;
+      const bool persistent = b->persist;
+      // Timed as stepping runs (graph replays for each kGraphSteps); an even count
+      // returns to the same slab, so the warm-up run captures the graph the timed run
+      // replays.
+      const int n_t = steps + (steps & 1);
+      rc = do_steps(b, n_t);  // warm-up
+      if (rc) break;
+      double per = -1.0;  // the better of two timed runs
+      for (int rep = 0; rep < 2; ++rep) {
+        if (!cu(cudaEventRecord(e0, b->stream), "cudaEventRecord")) break;
+        rc = do_steps(b, n_t);
         if (rc) break;
+        if (!cu(cudaEventRecord(e1, b->stream), "cudaEventRecord")) break;
+        if (!cu(cudaEventSynchronize(e1), "cudaEventSynchronize")) break;
+        float ms = 0.f;
+        if (!cu(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime")) break;
+        if (per < 0 || ms / n_t < per) per = ms / n_t;
       }
       if (rc) break;
+      if (best.ms < 0 || per < best.ms) {
+        best.nt = nt;
+        best.vec = vec;
+        best.rows = rows;
+        best.ms = per;
+        best.persist = persist;
+      }
+      if (!persistent) break;  // the tiling does not step persistently: timed once
     }
-    if (rc) break;
+  };
+  // the default's choice for a single lattice, whose height may lie between those below
+  if (b->n_inst == 1) {
+    b->nt_auto = true;
+    b->vec = default_vec(b->fp64);
+    b->rows_req = 0;
+    b->persist_off = false;
+    choose_tiling(b);
+    time_tiling(b->nt, b->vec, b->rows);
   }
+  for (int vec : vecs)
+    for (int nt : nts) {
+      if (!tiling_ok(b->fp64, nt, vec)) continue;
+      for (int rows : rows_c)
+        if (rc == LBM_OK) time_tiling(nt, vec, rows);
+    }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   // Restore the state into both slabs and the bookkeeping.
