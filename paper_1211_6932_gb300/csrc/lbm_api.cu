@@ -439,8 +439,8 @@ int persist_kind(const Batch* b, int* nt_out = nullptr) {
 // Whether chunks of `rows` rows give the active instances at least two waves of step items
 // (resident persistent CTAs): with fewer, a step's first items would wait on the previous
 // step's last ones, since the odd steps' lists start only half a step further on (the
-// 1024^2 ellipse, 640 items per step against 760 resident CTAs, stepped at 48 against 53
-// GLUPS persistently).
+// 1024^2 ellipse, 640 items per step against 760 resident CTAs, takes 16.7 us a step
+// persistently and 13.5 with a launch per step).
 bool persist_items_ok(const Batch* b, int rows) {
   int nt = 0;
   const int kind = persist_kind(b, &nt);
@@ -475,8 +475,8 @@ int default_rows(const Batch* b) {
   const int r6 = clamp((long long)std::ceil(sm_rows / ((double)std::max(b->sms, 1) * 6.0)));
   // Persistent stepping has no drain between steps, so fewer, taller chunks (fewer halo
   // rows) win: about three waves, rounded up to a multiple of four rows (32 rows at 4096^2,
-  // 87.5 against 84.0 GLUPS at 16 rows per step), if that still gives the two waves of
-  // items per step that persistent stepping needs (persist_items_ok).
+  // 182.8 us a step against 186.3 with 16 rows and a launch per step), if that still gives the
+  // two waves of items per step that persistent stepping needs (persist_items_ok).
   if (persist_allowed(b) && persist_kind(b) >= 0) {
     const long long r3 = (long long)std::ceil(sm_rows / ((double)std::max(b->sms, 1) * 3.0));
     const int rp = clamp((r3 + 3) / 4 * 4);
@@ -505,7 +505,11 @@ bool overlap_ok(long long items, int occ, int sms) {
 // start-up) a latency and the issue of the W warps that the busiest SM holds; with more items
 // than resident CTAs, the work itself.  Chunks used to be eight rows at least: 64 x 64 stepped
 // in 7.4 us and takes 2.3 with one-row chunks, 601 x 407 in 9.6 and 6.0, and 1024^2 in 17.2
-// (strips of 252 columns cover 1260) and 13.5 (six of 188 cover 1128).
+// (strips of 252 columns cover 1260) and 13.5 (six of 188 cover 1128).  Not used where the
+// default rule gives two waves of items (persist_items_ok), also if persistent stepping is
+// switched off: the launches then read and write far more than the L2 holds, which the model
+// does not know (4096^2 per step: 186 with the default's 16 rows, 210 with its 96 x 64;
+// 2048^2: 53 and 57).
 struct Tiling {
   int nt, rows;
 };
@@ -576,8 +580,7 @@ void choose_tiling(Batch* b) {
         b, b->nt_auto ? std::vector<int>{128, 64} : std::vector<int>{b->nt});
     b->nt = t.nt;
     b->rows = t.rows;
-  } else if (b->vec == 2 && persist_env() != 2 &&
-             !(persist_allowed(b) && persist_items_ok(b, b->rows))) {
+  } else if (b->vec == 2 && persist_env() != 2 && !persist_items_ok(b, b->rows)) {
     const Tiling t = choose_pair_tiling(
         b, b->nt_auto ? std::vector<int>{128, 96, 64, 32} : std::vector<int>{b->nt});
     b->nt = t.nt;
