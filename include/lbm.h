@@ -199,7 +199,9 @@ int lbm_step(lbm_handle* h, int n);
  * item taking the sweep of its instance), at least two waves of work items per step (with
  * fewer, the first items of a step would wait on the last ones of the step before), when
  * every work item depends on at most four chunk rows (chunks of two rows or more), unless the
- * autotuner measured one launch per step faster for the tiling it chose, and unless the
+ * autotuner measured one launch per step faster for the tiling it chose, unless a batch at
+ * its default tiling has three tenths of its nodes or more in either kind of strips (two
+ * launches per step are faster then; LBM_PERSISTENT=1 keeps the one), and unless the
  * environment sets LBM_PERSISTENT=0 when the work lists are built (creation, tiling
  * change, retirement); LBM_PERSISTENT=2 drops the two-wave condition (for tests).  With it
  * the default chunk height aims at about three waves of CTAs instead of six (taller

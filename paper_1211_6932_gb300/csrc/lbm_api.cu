@@ -404,8 +404,8 @@ bool transposed_layout(const lbm_instance& in, int nt, int vec) {
 int step_nt(const Batch* b, int i) { return per_instance(b) ? b->inst_nt[i] : b->nt; }
 
 // LBM_PERSISTENT in the environment: 0 never steps persistently, 2 whenever the
-// dependency rule allows (even with few items per step; for tests), anything else (the
-// default) when there are enough items per step.
+// dependency rule allows (even with few items per step; for tests), 1 when there are enough
+// items per step, and unset the same but for some batches of both kinds (branches_better).
 int persist_env() {
   const char* env = std::getenv("LBM_PERSISTENT");
   return env ? std::atoi(env) : 1;
@@ -451,6 +451,28 @@ bool persist_items_ok(const Batch* b, int rows) {
       items += (long long)lbm::strips_for(b->inst[i].nx, nt, b->vec) *
                ((b->inst[i].ny + rows - 1) / rows);
   return items >= 2LL * lbm::persist_occupancy(b->rule, nt, kind) * std::max(b->sms, 1);
+}
+
+// Whether a batch of both kinds of strips at its default tiling steps with one launch per step
+// and kind instead: if each kind has at least three tenths of the nodes, the two branches fill
+// each other's last waves, and each kernel keeps its five CTAs an SM where the common one has
+// four.  us per step as one persistent launch and as two branches (same chunk heights), by the
+// strips' share of the nodes: 0.64 (256 instances of sides 64 to 512) 163.5 and 155.9, 0.69
+// 115.6 and 110.3, 0.59 51.7 and 48.1, 0.53 59.4 and 57.6, 0.45 84.9 and 82.6, 0.33 104.7 and
+// 100.9; but 0.91 97.8 and 107.2, 0.15 68.8 and 69.7, 0.13 49.8 and 52.1.  LBM_PERSISTENT=1
+// keeps the one launch; a tiling asked for (or chosen by the autotuner, which times both) does
+// too.
+bool branches_better(const Batch* b, int kind) {
+  if (kind != lbm::PERSIST_MIXED || b->rows_req > 0 || std::getenv("LBM_PERSISTENT")) return false;
+  long long strip = 0, all = 0;
+  for (int i = 0; i < b->n_inst; ++i)
+    if (b->active[i]) {
+      const InstParams& P = b->inst[i];
+      const long long n = (long long)P.nx * P.ny;
+      all += n;
+      if (!lbm::full_width(P.nx, step_nt(b, i), b->vec)) strip += n;
+    }
+  return 10 * strip >= 3 * all && 10 * (all - strip) >= 3 * all;
 }
 
 // Rows per CTA sweep: about six waves of resident CTAs (measured best on 4096^2: fewer
@@ -709,6 +731,8 @@ bool plan_persist_list(const std::vector<WorkItem>& items, int lo, int hi,
   return true;
 }
 
+int ensure_branches(Batch* b);
+
 int build_persist(Batch* b) {
   b->persist = false;
   int nt = 0;
@@ -716,6 +740,7 @@ int build_persist(Batch* b) {
   if (!persist_allowed(b) || b->n_items == 0 || kind < 0 ||
       (persist_env() != 2 && !persist_items_ok(b, b->rows)))
     return LBM_OK;
+  if (branches_better(b, kind)) return ensure_branches(b);
   const int n = b->n_items;
   std::vector<WorkItem> items2(2 * (size_t)n);
   std::vector<ItemLink> links2(2 * (size_t)n);

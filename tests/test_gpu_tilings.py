@@ -29,3 +29,36 @@ def test_default_tiling_equals_eight_row_chunks(walls):
                 got.append(L.get_populations())
         for g in got[1:]:
             assert np.array_equal(got[0], g), (nx, ny)
+
+
+@pytest.mark.parametrize("wide,narrow,branches", [(12, 40, True), (14, 4, False), (2, 110, False)])
+def test_batches_of_both_kinds_of_strips_choose_their_stepping(monkeypatch, wide, narrow, branches):
+    """At the default tiling a batch with three tenths of its nodes or more in either kind steps
+    with a launch per step and kind, others as one persistent launch: same bits as with
+    LBM_PERSISTENT=1, which always takes the one launch, over runs with and without a graph."""
+    from paper_1211_6932_gb300 import Batch
+    from tests.test_gpu_batch import instance, start_fields
+    cs = [pairs.case(500, 420 + i % 3, tr=0.75, sigma=0.114) for i in range(wide)]
+    cs += [pairs.case(250 - i % 2, 250, tr=0.8, sigma=0.11) for i in range(narrow)]
+    fields = [start_fields(c, 60 + i) for i, c in enumerate(cs)]
+    got = []
+    for env in (None, "1"):
+        monkeypatch.delenv("LBM_PERSISTENT", raising=False)
+        if env:
+            monkeypatch.setenv("LBM_PERSISTENT", env)
+        b = Batch([instance(c) for c in cs], precision="fp32")
+        try:
+            for i, fl in enumerate(fields):
+                b.init_fields(i, *fl)
+            if env:
+                assert b.persistent and b.launches_per_step == 1
+            else:
+                assert b.persistent == (not branches)
+                assert b.launches_per_step == (2 if branches else 1)
+            b.step(70)
+            b.step(6)
+            got.append([b.get_populations(i) for i in range(0, len(cs), 7)])
+        finally:
+            b.close()
+    for x, y in zip(*got):
+        assert np.array_equal(x, y)
