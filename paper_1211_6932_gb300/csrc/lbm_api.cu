@@ -1175,10 +1175,12 @@ int do_steps(Batch* b, long long n) {
   if (n < 0) return set_err(b->err, LBM_EINVAL, "step count must be >= 0");
   if (b->n_items == 0) return LBM_OK;
   const long long n0 = n;
-  // Runs of kGraphSteps are replayed from a graph, and so are the powers of two of what is
-  // left, once a run of that length comes back (36 launches of a 100-step call kept the host
-  // busy for 80 us, more than the steps of a small lattice take); a persistent run of any
-  // length is one launch.
+  // Runs of kGraphSteps and of the lower powers of two are replayed from a graph once a run of
+  // that length comes back (36 launches of a 100-step call kept the host busy for 80 us, more
+  // than the steps of a small lattice take); a persistent run of any length is one launch.
+  // The first run is launched: the GPU steps while the host queues the launches, but waits
+  // for a capture (the first 100 steps of 193 x 147 with their transfers: 670 us with the
+  // capture, 381 without), and a batch that retires instances would wait at every retirement.
   // A caller's own capture of a short run gets its launches, as it did.
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(b->stream, &capture) != cudaSuccess) cudaGetLastError();
@@ -1186,8 +1188,7 @@ int do_steps(Batch* b, long long n) {
   while (n > 0) {
     int k = kGraphLog;
     while (k > 0 && (1LL << k) > n) --k;
-    const bool whole = k == kGraphLog;
-    if (whole || (k > 0 && replay && b->graph_uses[k][b->cur] > 0)) {
+    if (replay ? k > 0 && b->graph_uses[k][b->cur] > 0 : k == kGraphLog) {
       if (!b->graph[k][b->cur]) {
         int rc = capture_graph(b, k, b->cur);
         if (rc) return rc;
