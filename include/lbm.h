@@ -180,8 +180,8 @@ int lbm_get_populations(lbm_handle* h, double* f);
 /*
  * Advance n >= 0 time steps (Eqs. 1-7 with the forcing of Eq. 25, Sec. II-III).  Each
  * step is one pass of the fused kernel: one launch per step, or, stepping persistently
- * (see lbm_persistent), one launch per run of up to 64 steps; runs of 64 steps, and the
- * powers of two below once they come back, are replayed from a CUDA graph.
+ * (see lbm_persistent), one launch per run of up to 64 steps; runs of 64 steps and of the
+ * powers of two below are replayed from a CUDA graph once they come back.
  * Asynchronous: returns once the work is queued.  Status is reported by lbm_sync and by
  * every synchronous call.
  */
