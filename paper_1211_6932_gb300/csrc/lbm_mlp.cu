@@ -11,7 +11,7 @@
 //                     block's 8 warps (warp w sums rows w, w + 8, ... in order); the 8
 //                     partial sums are added in warp order (deterministic), then the
 //                     Adam update of the FP32 master weight, its moments and its BF16
-//                     copy.  Block 0 also reduces the loss in a fixed order.  (One thread
+//                     copy.  One more block reduces the loss in a fixed order.  (One thread
 //                     per parameter summing all rows left one warp per SM waiting on its
 //                     loads: 34 us of a 49 us update under ncu, against 18.6 us.  With 32
 //                     row slices the Adam trajectory of 60 updates left 1.4 % of the
@@ -89,6 +89,9 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // Programmatic dependent launch: wait until the preceding kernel of the stream has completed
 // (nothing to wait for after an ordinary launch), and let the following one be launched.
+// Whatever an update writes (weights, moments, counter, the rows' scratch), here or two
+// kernels back, is visible to a kernel only after its own wait: it is read behind it, and
+// through pointers that promise nothing about other writers (no const __restrict__).
 __device__ __forceinline__ void wait_predecessor() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -100,9 +103,9 @@ enum { ROWS_PREDICT = 0, ROWS_TRAIN = 1 };
 
 template <int MODE>
 __global__ void __launch_bounds__(ROWS_PER_BLOCK * 32) mlp_rows_kernel(
-    const __nv_bfloat16* __restrict__ w, const float* __restrict__ x,
+    const __nv_bfloat16* w, const float* __restrict__ x,
     const float* __restrict__ t, int n, Scaling sc, RowBufs rb, double* __restrict__ y_out,
-    long long* __restrict__ update_counter) {
+    long long* update_counter) {
   __shared__ float sW1[NH * W1S], sB1[NH], sW2[NH * W2S], sB2[NH], sW3[NO * NH], sB3[NO];
   __shared__ float sBuf[ROWS_PER_BLOCK][NH];
   const int tid = threadIdx.x;
@@ -266,10 +269,9 @@ __global__ void __launch_bounds__(ROWS_PER_BLOCK * 32) mlp_rows_kernel(
 enum { PARAM_GRAD = 0, PARAM_ADAM = 1 };
 
 __global__ void __launch_bounds__(PARAM_THREADS + 32) mlp_param_kernel(
-    RowBufs rb, int n, float* __restrict__ master, __nv_bfloat16* __restrict__ w,
-    float* __restrict__ m1, float* __restrict__ m2, float* __restrict__ grad_out, AdamArgs a,
-    int mode, const long long* __restrict__ update_counter, float* __restrict__ loss_hist,
-    float* __restrict__ loss_out) {
+    RowBufs rb, int n, float* master, __nv_bfloat16* w, float* m1, float* m2,
+    float* __restrict__ grad_out, AdamArgs a, int mode, const long long* update_counter,
+    float* __restrict__ loss_hist, float* __restrict__ loss_out) {
   const int tid = threadIdx.x;
   if (blockIdx.x == PARAM_BLOCKS) {
     // loss: fixed partition of the rows over the threads, then a fixed tree
@@ -298,14 +300,6 @@ __global__ void __launch_bounds__(PARAM_THREADS + 32) mlp_param_kernel(
   const int p = blockIdx.x * 32 + lane;
   __shared__ float part[PARAM_SLICES][32];
   __shared__ float bias1, bias2;  // 1 - beta^k
-  // the last update's moments and weight: that kernel has completed before this one's
-  // predecessor lets it be launched
-  float old1 = 0.f, old2 = 0.f, oldw = 0.f;
-  if (slice == 0 && p < NP && mode == PARAM_ADAM) {
-    old1 = m1[p];
-    old2 = m2[p];
-    oldw = master[p];
-  }
   // dL/dp = sum over rows of (delta of the output unit) x (input value): warp `slice` sums
   // rows slice, slice + PARAM_SLICES, ... in order, lane l for parameter p
   const float* da = nullptr;
@@ -326,6 +320,13 @@ __global__ void __launch_bounds__(PARAM_THREADS + 32) mlp_param_kernel(
   }
   wait_predecessor();
   launch_dependents();
+  // the last update's moments and weight, in flight together with the rows' values
+  float old1 = 0.f, old2 = 0.f, oldw = 0.f;
+  if (slice == 0 && p < NP && mode == PARAM_ADAM) {
+    old1 = m1[p];
+    old2 = m2[p];
+    oldw = master[p];
+  }
   if (slice == PARAM_SLICES) {  // the last warp: Adam's bias corrections meanwhile
     if (mode == PARAM_ADAM && lane < 2) {
       const float k = (float)*update_counter;
