@@ -79,8 +79,8 @@ typedef struct {
   int precision;  /* LBM_FP32_DEV (default) or LBM_FP64 */
   int visc_mode;  /* -1 (default): LBM_VISC_STEP if nu_l > 0 and nu_v > 0, else CONST */
   int bc;         /* LBM_BC_PERIODIC (default) or LBM_BC_WALLS_Y */
-  int psi_fp64;   /* FP32_DEV only: 1 evaluates psi (Eqs. 24, 30) to double-precision accuracy
-                     (pairs of floats, 45 bits) and rounds it to float once */
+  int psi_fp64;   /* FP32_DEV only: 1 evaluates psi (Eqs. 24, 30) in double precision and rounds it
+                     to float once (in pairs of floats where they decide the rounding) */
   double rho_ref; /* FP32_DEV deviation reference; < 0 (default): the Maxwell vapour
                      density when T < T_c, else 0.  Ignored for LBM_FP64 (always 0). */
   double rho_c;   /* STEP switch density; <= 0 (default): 0.5218 / b (Sec. IV A) */

@@ -46,7 +46,7 @@ struct Batch {
   std::vector<char> tr;          // instance stored transposed (lbm_instance.layout)
   std::vector<int> active;
   // Viscosity rule of the pair kernel's steps (PAIR_ANY unless every instance has the same
-  // rule, b, G and rates) and the constants the instances share.
+  // rule, b, G and rates; PAIR_PSI64 with the psi_fp64 option) and the constants the instances share.
   int rule = lbm::PAIR_ANY;
   lbm::PairConsts shared{};
   // Tensor maps of the pair kernel's row copies, for the widths of the step launches and of
@@ -970,6 +970,7 @@ void set_rule(Batch* b) {
     for (int k = 0; k < lbm::Q; ++k) same &= P.s[k] == A.s[k];
     if (!same) b->rule = lbm::PAIR_ANY;
   }
+  if (A.psi_fp64) b->rule = lbm::PAIR_PSI64;  // single lattices only
   b->shared = lbm::pair_params(A);
 }
 
@@ -1066,7 +1067,7 @@ int launch_group(Batch* b, int g, int c, bool dependent, cudaStream_t st) {
                             (double*)b->slab[c ^ 1], b->d_inst, items, n, b->d_status, st);
   } else if (b->fp64) {
     MomArgs<double> mo{};
-    e = lbm::launch_sweep<double>(b->grp_nt[g], lbm::MODE_STEP, b->grp_full[g], (const double*)b->slab[c],
+    e = lbm::launch_sweep<double>(false, b->grp_nt[g], lbm::MODE_STEP, b->grp_full[g], (const double*)b->slab[c],
                                   (double*)b->slab[c ^ 1], b->d_inst, items, n, mo, b->d_status,
                                   st);
   } else if (b->vec == 2) {
@@ -1075,7 +1076,7 @@ int launch_group(Batch* b, int g, int c, bool dependent, cudaStream_t st) {
                          dependent, st);
   } else {
     MomArgs<float> mo{};
-    e = lbm::launch_sweep<float>(b->grp_nt[g], lbm::MODE_STEP, b->grp_full[g], (const float*)b->slab[c],
+    e = lbm::launch_sweep<float>(b->rule == lbm::PAIR_PSI64, b->grp_nt[g], lbm::MODE_STEP, b->grp_full[g], (const float*)b->slab[c],
                                  (float*)b->slab[c ^ 1], b->d_inst, items, n, mo, b->d_status,
                                  st);
   }
@@ -1452,12 +1453,12 @@ cudaError_t launch_moments(const Batch* b, const WorkItem* d_items, int n, const
     if (!kind[full]) continue;
     if constexpr (sizeof(S) == 4) {
       if (b->vec == 2) {
-        e = lbm::launch_pair_moments(mom_nt(b), full, b->maps_mom, b->cur, b->d_inst, d_items, n,
-                                     mo, b->d_status, b->stream);
+        e = lbm::launch_pair_moments(b->rule, mom_nt(b), full, b->maps_mom, b->cur, b->d_inst,
+                                     d_items, n, mo, b->d_status, b->shared, b->stream);
         continue;
       }
     }
-    e = lbm::launch_sweep<S>(mom_nt(b), lbm::MODE_MOMENTS, full, (const S*)b->slab[b->cur], nullptr,
+    e = lbm::launch_sweep<S>(b->rule == lbm::PAIR_PSI64, mom_nt(b), lbm::MODE_MOMENTS, full, (const S*)b->slab[b->cur], nullptr,
                              b->d_inst, d_items, n, mo, b->d_status, b->stream);
   }
   return e;

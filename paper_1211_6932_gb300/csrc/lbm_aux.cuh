@@ -119,7 +119,11 @@ __global__ void psi_kernel(const double* __restrict__ rho, double* __restrict__ 
   const Phys<S> ph = load_phys<S>(*Pp);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
-    out[i] = (double)psi_t<S, S>((S)rho[i], ph);
+    if constexpr (sizeof(S) == 4)
+      out[i] = (double)(Pp->psi_fp64 ? psi_fp64((S)rho[i], Pp->split, *Pp)
+                                     : psi_t<S, S>((S)rho[i], ph));
+    else
+      out[i] = psi_t<S, S>(rho[i], ph);
 }
 
 }  // namespace lbm

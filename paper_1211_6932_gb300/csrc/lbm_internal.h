@@ -9,9 +9,9 @@ namespace lbm {
 // Launch the fused one-column sweep (MODE_STEP) or its moments/diagnostics pass
 // (MODE_MOMENTS) over n_items work items with nt threads per CTA, in full-width strips or not
 // (see strips_for; a CTA of the moments pass whose instance is of the other kind returns at
-// once).
+// once); psi64: with the psi_fp64 option (FP32).
 template <typename S>
-cudaError_t launch_sweep(int nt, int mode, int full, const S* fin, S* fout, const InstParams* d_inst,
+cudaError_t launch_sweep(bool psi64, int nt, int mode, int full, const S* fin, S* fout, const InstParams* d_inst,
                          const WorkItem* d_items, int n_items, const MomArgs<S>& mo,
                          int* d_status, cudaStream_t st);
 // Step of FP64 items of one row each (short64_kernel), reading the given slab by row map.
@@ -21,13 +21,14 @@ cudaError_t launch_short64(int nt, int full, const RowMaps& maps, int slab, doub
 // Pair kernel (two columns per thread): the moments/diagnostics pass over the items of one
 // kind (full-width strips or not; a CTA whose instance is of the other kind returns at
 // once), and a step for a viscosity rule (VISC_* with the constants that the instances of the
-// launch share, or PAIR_ANY).  Both read the slab of the given index through the row maps.
+// launch share, PAIR_ANY or PAIR_PSI64).  Both read the slab of the given index through the row maps.
 // rows: the items' chunk height (one and two rows have a kernel of their own); dependent:
 // launched as a programmatic dependent of the stream's previous kernel, which must be the
 // previous step.
-cudaError_t launch_pair_moments(int nt, int full, const RowMaps& maps, int slab,
+cudaError_t launch_pair_moments(int rule, int nt, int full, const RowMaps& maps, int slab,
                                 const InstParams* d_inst, const WorkItem* d_items, int n_items,
-                                const MomArgs<float>& mo, int* d_status, cudaStream_t st);
+                                const MomArgs<float>& mo, int* d_status,
+                                const PairConsts& shared, cudaStream_t st);
 cudaError_t launch_pair(int rule, int nt, int rows, int full, const RowMaps& maps, int slab,
                         float* fout,
                         const InstParams* d_inst, const WorkItem* d_items, int n_items,

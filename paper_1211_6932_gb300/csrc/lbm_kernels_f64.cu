@@ -4,11 +4,11 @@
 namespace lbm {
 
 template <>
-cudaError_t launch_sweep<double>(int nt, int mode, int full, const double* fin, double* fout,
+cudaError_t launch_sweep<double>(bool, int nt, int mode, int full, const double* fin, double* fout,
                                  const InstParams* d_inst, const WorkItem* d_items, int n_items,
                                  const MomArgs<double>& mo, int* d_status, cudaStream_t st) {
-  if (nt == 64) return launch_sweep_mode<double, 64>(mode, full, fin, fout, d_inst, d_items, n_items, mo, d_status, st);
-  if (nt == 128) return launch_sweep_mode<double, 128>(mode, full, fin, fout, d_inst, d_items, n_items, mo, d_status, st);
+  if (nt == 64) return launch_sweep_mode<double, 64, false>(mode, full, fin, fout, d_inst, d_items, n_items, mo, d_status, st);
+  if (nt == 128) return launch_sweep_mode<double, 128, false>(mode, full, fin, fout, d_inst, d_items, n_items, mo, d_status, st);
   return cudaErrorInvalidValue;
 }
 

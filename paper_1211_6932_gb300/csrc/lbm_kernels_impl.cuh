@@ -40,43 +40,39 @@ static cudaError_t launch_kernel(void (*kernel)(P...), int blocks, int threads, 
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-template <typename S, int NT, int MODE, bool FULL>
+template <typename S, int NT, int MODE, bool FULL, bool PSI64>
 static cudaError_t launch_sweep_cfg(const S* fin, S* fout, const InstParams* d_inst,
                                     const WorkItem* d_items, int n_items, const MomArgs<S>& mo,
                                     int* d_status, cudaStream_t st) {
   constexpr size_t smem = SweepCfg<S, NT>::BYTES;
   static std::atomic<unsigned long long> done{0};
-  cudaError_t e = ensure_smem_attr(sweep_kernel<S, NT, MODE, FULL>, smem, done);
+  cudaError_t e = ensure_smem_attr(sweep_kernel<S, NT, MODE, FULL, PSI64>, smem, done);
   if (e != cudaSuccess) return e;
   if (n_items <= 0) return cudaSuccess;
-  sweep_kernel<S, NT, MODE, FULL><<<n_items, NT, smem, st>>>(fin, fout, d_inst, d_items, n_items,
-                                                       mo, d_status);
+  sweep_kernel<S, NT, MODE, FULL, PSI64><<<n_items, NT, smem, st>>>(fin, fout, d_inst, d_items,
+                                                                   n_items, mo, d_status);
   return cudaGetLastError();
 }
 
-template <typename S, int NT>
+template <typename S, int NT, bool PSI64>
 static cudaError_t launch_sweep_mode(int mode, int full, const S* fin, S* fout, const InstParams* d_inst,
                                      const WorkItem* d_items, int n_items,
                                      const MomArgs<S>& mo, int* d_status, cudaStream_t st) {
-  if (mode == MODE_STEP)
-    return full ? launch_sweep_cfg<S, NT, MODE_STEP, true>(fin, fout, d_inst, d_items, n_items,
-                                                           mo, d_status, st)
-                : launch_sweep_cfg<S, NT, MODE_STEP, false>(fin, fout, d_inst, d_items, n_items,
-                                                            mo, d_status, st);
-  return full ? launch_sweep_cfg<S, NT, MODE_MOMENTS, true>(fin, fout, d_inst, d_items, n_items,
-                                                            mo, d_status, st)
-              : launch_sweep_cfg<S, NT, MODE_MOMENTS, false>(fin, fout, d_inst, d_items, n_items,
-                                                             mo, d_status, st);
+#define LBM_SWEEP(M, F)                                                                         \
+  launch_sweep_cfg<S, NT, M, F, PSI64>(fin, fout, d_inst, d_items, n_items, mo, d_status, st)
+  if (mode == MODE_STEP) return full ? LBM_SWEEP(MODE_STEP, true) : LBM_SWEEP(MODE_STEP, false);
+  return full ? LBM_SWEEP(MODE_MOMENTS, true) : LBM_SWEEP(MODE_MOMENTS, false);
+#undef LBM_SWEEP
 }
 
 template <typename S, int NT>
 static int occupancy_cfg() {
   constexpr size_t smem = SweepCfg<S, NT>::BYTES;
-  cudaFuncSetAttribute(sweep_kernel<S, NT, MODE_STEP, false>,
+  cudaFuncSetAttribute(sweep_kernel<S, NT, MODE_STEP, false, false>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int occ = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &occ, sweep_kernel<S, NT, MODE_STEP, false>, NT, smem);
+      &occ, sweep_kernel<S, NT, MODE_STEP, false, false>, NT, smem);
   return (e == cudaSuccess && occ > 0) ? occ : 1;
 }
 

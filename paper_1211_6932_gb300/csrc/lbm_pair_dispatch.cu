@@ -9,6 +9,7 @@ namespace lbm {
     case VISC_CONST: return FN<VISC_CONST>(__VA_ARGS__);                           \
     case VISC_STEP: return FN<VISC_STEP>(__VA_ARGS__);                             \
     case VISC_LINEAR: return FN<VISC_LINEAR>(__VA_ARGS__);                         \
+    case PAIR_PSI64: return FN<PAIR_PSI64>(__VA_ARGS__);                           \
     default: return FN<PAIR_ANY>(__VA_ARGS__);                                     \
   }
 

@@ -1,5 +1,5 @@
 // Launchers of the FP32 pair kernel (two columns per thread, packed float2 arithmetic) for
-// one viscosity rule (VISC_* or PAIR_ANY), one translation unit per rule.
+// one viscosity rule (VISC_*, PAIR_ANY or PAIR_PSI64), one translation unit per rule.
 #pragma once
 #include "lbm_kernels_impl.cuh"
 
