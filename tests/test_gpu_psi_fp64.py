@@ -24,15 +24,23 @@ def wide_psi(rho, c):
         return np.where(arg > 0, np.sqrt(arg), L(0)), ratio
 
 
+def vanishing_density(c):
+    """The density in (0.3, 0.9) above which psi is 0, by bisection."""
+    lo, hi = 0.3, 0.9
+    assert wide_psi(np.array([lo]), c)[0] > 0 and wide_psi(np.array([hi]), c)[0] == 0
+    while hi - lo > 1e-13:
+        mid = 0.5 * (lo + hi)
+        lo, hi = (mid, hi) if wide_psi(np.array([mid]), c)[0][0] > 0 else (lo, mid)
+    return lo
+
+
 def densities(c):
     """Floats over the whole range of use, up to and beyond x = 3/4, dense next to psi = 0."""
     rng = np.random.default_rng(5)
-    x = np.linspace(0.3, 0.9, 20001)
-    p, _ = wide_psi(x, c)
-    k = int(np.argmax((p[:-1] > 0) & (p[1:] == 0)))  # psi vanishes between x[k] and x[k + 1]
+    zero = vanishing_density(c)
     rho = np.concatenate([np.exp(rng.uniform(np.log(1e-4), np.log(0.9), 400000)),
                           np.geomspace(1e-38, 1e-4, 20000),
-                          rng.uniform(x[k] - 1e-3, x[k + 1], 200000)])
+                          rng.uniform(zero - 1e-3, zero, 200000)])
     return np.unique(rho.astype(np.float32)).astype(np.float64)
 
 
@@ -74,10 +82,7 @@ def test_where_fp64_decides():
 
 def vanishing(c, shape, seed):
     """Columns of densities at psi = 0 (floats within 1e-6 below it) between columns of 0.1."""
-    x = np.linspace(0.3, 0.74, 4000001)
-    p, _ = wide_psi(x, c)
-    k = int(np.argmax((p[:-1] > 0) & (p[1:] == 0)))
-    rho = x[k] - np.random.default_rng(seed).uniform(0.0, 1e-6, shape)
+    rho = vanishing_density(c) - np.random.default_rng(seed).uniform(0.0, 1e-6, shape)
     rho = np.where(np.arange(shape[1])[None, :] % 3 == 0, 0.1, rho)
     return rho.astype(np.float32).astype(np.float64)
 
@@ -97,9 +102,10 @@ def test_plain_fp32_psi_misses_where_psi_vanishes():
 
 @gpu
 @pytest.mark.parametrize("walls", [False, True])
-@pytest.mark.parametrize("nx,vec,rows", [(96, 2, 1), (96, 2, 2), (96, 2, 7), (300, 2, 1),
-                                         (300, 2, 5), (96, 1, 4), (300, 1, 4)])
-def test_step_uses_it(nx, vec, rows, walls):
+@pytest.mark.parametrize("nx,vec,rows,persistent", [
+    (96, 2, 1, 0), (96, 2, 2, 0), (96, 2, 7, 0), (300, 2, 1, 0), (300, 2, 5, 0), (96, 1, 4, 0),
+    (300, 1, 4, 0), (96, 2, 7, 2), (300, 2, 5, 2)])
+def test_step_uses_it(monkeypatch, nx, vec, rows, persistent, walls):
     """One step of a lattice whose nodes hold rest populations only, so that FP32 sums them to
     the density exactly: with the option the step's error is that of its FP32 collision, some 30
     roundings of values up to the density (2^-24 each); plain FP32 psi, wrong by 1e-4 between
@@ -111,9 +117,11 @@ def test_step_uses_it(nx, vec, rows, walls):
     f[0] = rho
     ref = oracle.run(pairs.oracle_params(c), f, 1)
     err = {}
+    monkeypatch.setenv("LBM_PERSISTENT", str(persistent))
     for opt in (True, False):
         with pairs.gpu_lattice(c, "fp32", psi_fp64=opt, tile_vec=vec, tile_rows=rows,
                                rho_ref=0.0) as L:
+            assert L.persistent == (persistent == 2)
             L.set_populations(f)
             L.step(1)
             err[opt] = np.max(np.abs(L.get_populations() - ref))
