@@ -72,11 +72,12 @@ __global__ void __launch_bounds__(kFillThreads) fill_droplets_kernel(
       for (int j = 0; j < kTileNodes; ++j) {
         double dy = fabs((double)(yt + j * (kTileY / kTileNodes)) - d.cy);
         dy = fmin(dy, (double)ny - dy);
-        const double s = sqrt(dx * dx + dy * dy) - d.r_half;
+        const double s = sqrt(::fma(dx, dx, dy * dy)) - d.r_half;
         if (s > reach) continue;
         const double t = 2.0 * s / width;
-        const double v = 0.5 * (d.rho_in + rho_v) -
-                         0.5 * (d.rho_in - rho_v) * (t < -20.0 ? -1.0 : tanh(t));
+        // rounded before it is subtracted, whatever the compiler contracts around it
+        const double fall = __dmul_rn(0.5 * (d.rho_in - rho_v), t < -20.0 ? -1.0 : tanh(t));
+        const double v = 0.5 * (d.rho_in + rho_v) - fall;
         best[j] = fmax(best[j], v);
       }
     }
