@@ -21,7 +21,7 @@
 //
 // An update is a chain of latencies, not work: 256 rows are 7 MFLOP.  Both kernels are
 // launched as programmatic dependents, so that a kernel's launch and whatever does not need
-// its predecessor's results overlap the predecessor; a block has two rows, so that 256 rows
+// its predecessor's results overlap the predecessor; a training block has two rows, so that 256 rows
 // use 128 SMs and two warps share a block's shared-memory reads instead of eight; weights are
 // staged with 16-byte loads issued together; the bias corrections and the loss have a warp and
 // a block of their own.  256 rows: 18.9 us an update before, 7.3 now, with the same sums in
@@ -46,7 +46,10 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + NH * NI, OFF_W2 = OFF_B1 + NH,
 static_assert(OFF_B3 + NO == NP, "parameter packing");
 constexpr int W1S = NI + 1;  // padded row strides in shared memory
 constexpr int W2S = NH + 1;
-constexpr int ROWS_PER_BLOCK = 2;  // warps per block in the rows kernel
+// Warps, and so rows, per block of the rows kernel.  Predictions stage the weights for eight: us
+// a call with 2 and with 8 rows a block, 256 rows 35 and 35, 4096 52 and 51, 16384 100 and 87,
+// 65536 251 and 225.
+constexpr int TRAIN_ROWS = 2, PREDICT_ROWS = 8;
 constexpr int PARAM_SLICES = 8;    // row slices (warps) per parameter
 constexpr int PARAM_THREADS = 32 * PARAM_SLICES;
 constexpr int PARAM_BLOCKS = (NP + 31) / 32;      // 32 parameters per block
@@ -102,15 +105,16 @@ __device__ __forceinline__ void launch_dependents() {
 enum { ROWS_PREDICT = 0, ROWS_TRAIN = 1 };
 
 template <int MODE>
-__global__ void __launch_bounds__(ROWS_PER_BLOCK * 32) mlp_rows_kernel(
+__global__ void __launch_bounds__((MODE == ROWS_TRAIN ? TRAIN_ROWS : PREDICT_ROWS) * 32) mlp_rows_kernel(
     const __nv_bfloat16* w, const float* __restrict__ x,
     const float* __restrict__ t, int n, Scaling sc, RowBufs rb, double* __restrict__ y_out,
     long long* update_counter) {
+  constexpr int ROWS = MODE == ROWS_TRAIN ? TRAIN_ROWS : PREDICT_ROWS;
   __shared__ float sW1[NH * W1S], sB1[NH], sW2[NH * W2S], sB2[NH], sW3[NO * NH], sB3[NO];
-  __shared__ float sBuf[ROWS_PER_BLOCK][NH];
+  __shared__ float sBuf[ROWS][NH];
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
-  const int row = blockIdx.x * ROWS_PER_BLOCK + warp;
+  const int row = blockIdx.x * ROWS + warp;
   float xn[NI], tn[NO];
   if (row < n) {
 #pragma unroll
@@ -126,11 +130,11 @@ __global__ void __launch_bounds__(ROWS_PER_BLOCK * 32) mlp_rows_kernel(
   static_assert(OFF_B1 % 8 == 0 && OFF_W2 % 8 == 0 && OFF_B2 % 8 == 0 && OFF_W3 % 8 == 0 &&
                     OFF_B3 % 8 == 0 && NH % 8 == 0 && 8 % NI == 0,
                 "groups of eight weights");
-  constexpr int GROUPS = OFF_B3 / 8, PER = (GROUPS + ROWS_PER_BLOCK * 32 - 1) / (ROWS_PER_BLOCK * 32);
+  constexpr int GROUPS = OFF_B3 / 8, PER = (GROUPS + ROWS * 32 - 1) / (ROWS * 32);
   uint4 v[PER];
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
-    const int g = tid + k * ROWS_PER_BLOCK * 32;
+    const int g = tid + k * ROWS * 32;
     if (g < GROUPS) v[k] = reinterpret_cast<const uint4*>(w)[g];
   }
   if (tid < NO) sB3[tid] = __bfloat162float(w[OFF_B3 + tid]);
@@ -138,7 +142,7 @@ __global__ void __launch_bounds__(ROWS_PER_BLOCK * 32) mlp_rows_kernel(
   launch_dependents();
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
-    const int i = (tid + k * ROWS_PER_BLOCK * 32) * 8;
+    const int i = (tid + k * ROWS * 32) * 8;
     if (i >= OFF_B3) continue;
     float f[8];
     const __nv_bfloat162* h2v = reinterpret_cast<const __nv_bfloat162*>(&v[k]);
@@ -461,13 +465,14 @@ cudaError_t launch_dependent(void (*kernel)(P...), int blocks, int threads, cuda
 
 int launch_rows(lbm_mlp* h, int mode, int n, double* y_out, long long* counter,
                 cudaStream_t st) {
-  const int blocks = (n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK;
+  const int rows = mode == ROWS_TRAIN ? TRAIN_ROWS : PREDICT_ROWS;
+  const int blocks = (n + rows - 1) / rows;
   if (mode == ROWS_TRAIN)
-    MCK(h, launch_dependent(mlp_rows_kernel<ROWS_TRAIN>, blocks, ROWS_PER_BLOCK * 32, st, h->w,
-                            h->x, h->t, n, h->sc, h->rb, y_out, counter));
+    MCK(h, launch_dependent(mlp_rows_kernel<ROWS_TRAIN>, blocks, rows * 32, st, h->w, h->x, h->t, n,
+                            h->sc, h->rb, y_out, counter));
   else
-    mlp_rows_kernel<ROWS_PREDICT><<<blocks, ROWS_PER_BLOCK * 32, 0, st>>>(
-        h->w, h->xp, nullptr, n, h->sc, h->rb, y_out, counter);
+    mlp_rows_kernel<ROWS_PREDICT><<<blocks, rows * 32, 0, st>>>(h->w, h->xp, nullptr, n, h->sc,
+                                                               h->rb, y_out, counter);
   MCK(h, cudaGetLastError());
   return LBM_OK;
 }
