@@ -26,6 +26,7 @@
 #include "../../include/lbm.h"
 #include "../../include/lbm_warm.h"
 #include "lbm_internal.h"
+#include "lbm_runs.h"
 
 using lbm::InstParams;
 using lbm::MomArgs;
@@ -34,8 +35,7 @@ using lbm::WorkItem;
 
 namespace {
 
-constexpr int kGraphLog = 6;
-constexpr int kGraphSteps = 1 << kGraphLog;  // even, so a replay returns to the same slab
+using lbm::kGraphLog;
 thread_local std::string g_thread_err;
 
 struct Batch {
@@ -123,6 +123,7 @@ struct Batch {
   // that many steps has been queued launch by launch.
   cudaGraphExec_t graph[kGraphLog + 1][2] = {};
   int graph_uses[kGraphLog + 1][2] = {};
+  long long first_runs = 0;  // see queue_runs
   // Buffers allocated with guard bands (lbm_check_guards): base pointer, user bytes, name.
   struct Guarded {
     char* base;
@@ -1173,41 +1174,34 @@ int capture_graph(Batch* b, int k, int start) {
   return LBM_OK;
 }
 
+// The operations of queue_runs on a batch's stream.
+struct RunOps {
+  Batch* b;
+  int& uses(int k) { return b->graph_uses[k][b->cur]; }
+  bool captured(int k) { return b->graph[k][b->cur] != nullptr; }
+  long long& firsts() { return b->first_runs; }
+  int capture(int k) { return capture_graph(b, k, b->cur); }
+  int replay(int k) {
+    CK(b, cudaGraphLaunch(b->graph[k][b->cur], b->stream));
+    return LBM_OK;
+  }
+  int launch(int steps) {
+    int rc = queue_steps(b, steps, b->stream);
+    if (rc == LBM_OK) b->cur ^= steps & 1;
+    return rc;
+  }
+};
+
 int do_steps(Batch* b, long long n) {
   if (n < 0) return set_err(b->err, LBM_EINVAL, "step count must be >= 0");
   if (b->n_items == 0) return LBM_OK;
-  const long long n0 = n;
-  // Runs of kGraphSteps and of the lower powers of two are replayed from a graph once a run of
-  // that length comes back (36 launches of a 100-step call kept the host busy for 80 us, more
-  // than the steps of a small lattice take); a persistent run of any length is one launch.
-  // The first run is launched: the GPU steps while the host queues the launches, but waits
-  // for a capture (the first 100 steps of 193 x 147 with their transfers: 670 us with the
-  // capture, 381 without), and a batch that retires instances would wait at every retirement.
-  // A caller's own capture of a short run gets its launches, as it did.
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(b->stream, &capture) != cudaSuccess) cudaGetLastError();
-  const bool replay = !b->persist && capture == cudaStreamCaptureStatusNone;
-  while (n > 0) {
-    int k = kGraphLog;
-    while (k > 0 && (1LL << k) > n) --k;
-    if (replay ? k > 0 && b->graph_uses[k][b->cur] > 0 : k == kGraphLog) {
-      if (!b->graph[k][b->cur]) {
-        int rc = capture_graph(b, k, b->cur);
-        if (rc) return rc;
-      }
-      CK(b, cudaGraphLaunch(b->graph[k][b->cur], b->stream));
-      n -= 1LL << k;
-    } else {
-      const int m = b->persist ? (int)n : 1 << k;
-      int rc = queue_steps(b, m, b->stream);
-      if (rc) return rc;
-      ++b->graph_uses[k][b->cur];
-      b->cur ^= m & 1;
-      n -= m;
-    }
-  }
+  RunOps ops{b};
+  int rc = lbm::queue_runs(n, b->persist, capture != cudaStreamCaptureStatusNone, ops);
+  if (rc) return rc;
   for (int i = 0; i < b->n_inst; ++i)
-    if (b->active[i]) b->steps[i] += n0;
+    if (b->active[i]) b->steps[i] += n;
   return LBM_OK;
 }
 
@@ -1898,11 +1892,11 @@ int autotune(Batch* b, int steps, const char* cache_path, TileChoice& best) {
       rc = apply_tiling(b, nt, vec, rows, persist != 0);
       if (rc) break;
       const bool persistent = b->persist;
-      // Timed as stepping runs (graph replays for each kGraphSteps); an even count
-      // returns to the same slab, so the warm-up run captures the graph the timed run
-      // replays.
+      // Timed as stepping runs; an even count returns to the same slab, so once a warm-up run
+      // has been all replays (or one persistent launch), both timed runs are.
       const int n_t = steps + (steps & 1);
-      rc = do_steps(b, n_t);  // warm-up
+      RunOps ops{b};
+      rc = lbm::warm_up([&] { return do_steps(b, n_t); }, ops);
       if (rc) break;
       double per = -1.0;  // the better of two timed runs
       for (int rep = 0; rep < 2; ++rep) {
