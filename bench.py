@@ -10,7 +10,8 @@ flush is needed between steps.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
-Prints one JSON line (rank 0).  --impl reference times the FP64 CPU oracle on the host
+Prints one JSON line (rank 0); the studies beside it (other workloads, coexistence, precision,
+warm start and so on) go to stderr, a line each.  --impl reference times the FP64 CPU oracle on the host
 cores instead (each step: one oracle step on a 1024 x 1024 window of the same field).
 """
 import argparse
@@ -361,6 +362,7 @@ def run_batch(args):
     for _ in range(args.warmup):
         b.step(1)
     b.step(64)
+    b.step(64)  # captures the graph
     b.diagnostics()
     K = args.steps
     e0 = torch.cuda.Event(enable_timing=True)
@@ -456,9 +458,10 @@ def run_gpu(args):
     L.init_fields(rho)
     n_nodes = NX * NY
 
-    # warm-up (graph capture happens here)
+    # warm-up (a graph is captured when a run of its length comes back)
     for _ in range(args.warmup):
         L.step(1)
+    L.step(64)
     L.step(64)
     L.diagnostics()
     L.sync()
@@ -576,54 +579,20 @@ def run_gpu(args):
                                          "peak_source": "nominal FP64 rate",
                                          "fp64_flops_per_lu": flops}
         print("gpu part: %s" % json.dumps(line), file=sys.stderr, flush=True)
-        if not args.no_other_workloads and world == 1 and NX == 4096:
-            try:
-                line["other_workloads"] = other_workloads(stream)
-            except Exception as exc:  # reported, never hidden
-                line["other_workloads"] = {"error": repr(exc)}
-            print("other workloads: %s" % json.dumps(line["other_workloads"]), file=sys.stderr,
-                  flush=True)
-        if not args.no_other_workloads and world == 1 and NX == 4096:
-            try:
-                line["coexistence"] = coexistence_summary(stream)
-            except Exception as exc:  # reported, never hidden
-                line["coexistence"] = {"error": repr(exc)}
-            try:
-                line["interface"] = interface_summary(stream)
-            except Exception as exc:  # reported, never hidden
-                line["interface"] = {"error": repr(exc)}
-            try:
-                line["stability"] = stability_summary(stream)
-            except Exception as exc:  # reported, never hidden
-                line["stability"] = {"error": repr(exc)}
-            try:
-                line["calibration"] = calibration_summary(stream)
-            except Exception as exc:  # reported, never hidden
-                line["calibration"] = {"error": repr(exc)}
-            try:
-                line["dynamics"] = dynamics_summary(stream)
-            except Exception as exc:  # reported, never hidden
-                line["dynamics"] = {"error": repr(exc)}
-        if not args.no_other_workloads and world == 1 and NX == 4096:
-            try:
-                line["batch_equilibrium"] = batch_equilibrium_summary(stream)
-            except Exception as exc:  # reported, never hidden
-                line["batch_equilibrium"] = {"error": repr(exc)}
-            print("batch equilibrium: %s" % json.dumps(line["batch_equilibrium"]),
-                  file=sys.stderr, flush=True)
-        if not args.no_precision and world == 1 and NX == 4096:
-            try:
-                line["precision_error"] = precision_summary(stream)
-            except Exception as exc:  # reported, never hidden
-                line["precision_error"] = {"error": repr(exc)}
-            print("precision: %s" % json.dumps(line["precision_error"]), file=sys.stderr,
-                  flush=True)
-        if not args.no_warm_start and world == 1 and NX == 4096:
-            try:
-                line["warm_start"] = warm_start_ab(stream)
-            except Exception as exc:  # reported, never hidden
-                line["warm_start"] = {"error": repr(exc)}
-            print("warm start: %s" % json.dumps(line["warm_start"]), file=sys.stderr, flush=True)
+        if world == 1 and NX == 4096:
+            if not args.no_other_workloads:
+                for name, study in (("other_workloads", other_workloads),
+                                    ("coexistence", coexistence_summary),
+                                    ("interface", interface_summary),
+                                    ("stability", stability_summary),
+                                    ("calibration", calibration_summary),
+                                    ("dynamics", dynamics_summary),
+                                    ("batch_equilibrium", batch_equilibrium_summary)):
+                    report(name, study, stream)
+            if not args.no_precision:
+                report("precision_error", precision_summary, stream)
+            if not args.no_warm_start:
+                report("warm_start", warm_start_ab, stream)
         if not args.no_cpu_baseline:
             try:
                 line["cpu_baseline"] = cpu_baseline()[0]
@@ -635,6 +604,17 @@ def run_gpu(args):
         import torch.distributed as dist
         dist.destroy_process_group()
     return 0
+
+
+def report(name, study, *args):
+    """Run one of the studies beside the benchmark and print its JSON object to stderr as
+    "name: {...}": the benchmark's own line on stdout stays short enough to be read whole from
+    the end of a log."""
+    try:
+        result = study(*args)
+    except Exception as exc:  # reported, never hidden
+        result = {"error": repr(exc)}
+    print("%s: %s" % (name, json.dumps(result)), file=sys.stderr, flush=True)
 
 
 def other_workloads(stream):
@@ -655,6 +635,7 @@ def other_workloads(stream):
             L.autotune(steps=64)
         L.step(3)
         L.step(64)
+        L.step(64)  # captures the graph
         L.sync()
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
@@ -703,14 +684,14 @@ def other_workloads(stream):
         L.init_fields(rho, ux, uy)
         timed("splash_2048x512_walls_fp32", L, 2000, 2048 * 512, "f32", 72,
               "75 MB of state: L2-resident; autotuned tiling", tune=True)
-    # the 4096^2 field, FP32 storage with psi of Eq. 24 evaluated in FP64 (psi_fp64 option)
+    # the 4096^2 field, FP32 storage with psi of Eq. 24 to double precision (psi_fp64 option)
     e = Eos(a=A, T=eos_T(), b=B, R=R)
     rl, rv = maxwell(e)
     with Lattice(NX, NY, e, sigma=SIGMA, s=RATES, nu_l=NU_L, nu_v=NU_V, visc_mode="linear",
                  precision="fp32", psi_fp64=True, stream=stream) as L:
         L.init_fields(field(rl, rv))
         timed("droplets64_%dx%d_fp32_psi_fp64" % (NX, NY), L, 500, NX * NY, "f32", 72,
-              "FP32 storage and arithmetic, psi in FP64")
+              "FP32 storage and arithmetic, psi to double precision")
     # the 4096^2 field in the FP64 parity mode
     e = Eos(a=A, T=eos_T(), b=B, R=R)
     rl, rv = maxwell(e)
