@@ -200,7 +200,7 @@ int lbm_step(lbm_handle* h, int n);
  * fewer, the first items of a step would wait on the last ones of the step before), when
  * every work item depends on at most four chunk rows (chunks of two rows or more), unless the
  * autotuner measured one launch per step faster for the tiling it chose, unless a batch at
- * its default tiling has three tenths of its nodes or more in either kind of strips (two
+ * its default tiling has three tenths of its nodes or more in each kind of strips (two
  * launches per step are faster then; LBM_PERSISTENT=1 keeps the one), and unless the
  * environment sets LBM_PERSISTENT=0 when the work lists are built (creation, tiling
  * change, retirement); LBM_PERSISTENT=2 drops the two-wave condition (for tests).  With it

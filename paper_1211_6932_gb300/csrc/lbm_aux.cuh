@@ -121,9 +121,9 @@ __global__ void psi_kernel(const double* __restrict__ rho, double* __restrict__ 
        i += (long long)gridDim.x * blockDim.x)
     if constexpr (sizeof(S) == 4)
       out[i] = (double)(Pp->psi_fp64 ? psi_fp64((S)rho[i], Pp->split, *Pp)
-                                     : psi_t<S, S>((S)rho[i], ph));
+                                     : psi_t((S)rho[i], ph));
     else
-      out[i] = psi_t<S, S>(rho[i], ph);
+      out[i] = psi_t(rho[i], ph);
 }
 
 }  // namespace lbm

@@ -5,7 +5,8 @@
 // the host queues the launches, but waits for a capture (the first 100 steps of 193 x 147
 // with their transfers: 670 us with the capture, 381 without), and a batch that retires
 // instances would wait at every retirement.  The second run captures; from the third on a run
-// is a replay.  A caller's own capture of a short run gets its launches.
+// is a replay.  A caller's own capture of a short run gets its launches; of 64 steps and more it
+// fails, as no graph can be launched into a capture.
 #pragma once
 
 namespace lbm {
