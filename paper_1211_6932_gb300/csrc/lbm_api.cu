@@ -958,7 +958,7 @@ int fill_params(std::string& err, InstParams& P, const lbm_instance& in, bool fp
   P.rho_ref = fp64 ? 0.0 : (in.rho_ref >= 0 ? in.rho_ref : (have_maxwell ? mv : 0.0));
   fill_mirror(P.pf, P);
   fill_mirror(P.pd, P);
-  P.split = lbm::psi_split(P.b4, P.RT, P.a, P.two_over_G);
+  if (P.psi_fp64) P.split = lbm::psi_split(P.b4, P.RT, P.a, P.two_over_G);
   return LBM_OK;
 }
 
