@@ -1435,27 +1435,28 @@ int get_pops(Batch* b, int i, double* f) {
 }
 
 // Launch the moments/diagnostics kernel over a device list of n items on the batch's
-// stream.  The kernels have strip and full-width instantiations: both are launched over
-// the whole list, and each CTA works only on an item of its own kind.
+// stream.  The kernels have strip and full-width instantiations: of the pair kernel both are
+// launched over the whole list, and each CTA works only on an item of its own kind; the
+// one-column kernel has a third, for lists of both.
 template <typename S>
 cudaError_t launch_moments(const Batch* b, const WorkItem* d_items, int n, const MomArgs<S>& mo) {
   bool kind[2] = {false, false};  // strips, full-width strips present
   for (int i = 0; i < b->n_inst; ++i)
     kind[lbm::full_width(b->inst[i].nx, mom_nt(b), b->vec) ? 1 : 0] = true;
-  cudaError_t e = cudaSuccess;
-  for (int full = 0; full < 2 && e == cudaSuccess; ++full) {
-    if (!kind[full]) continue;
-    if constexpr (sizeof(S) == 4) {
-      if (b->vec == 2) {
-        e = lbm::launch_pair_moments(b->rule, mom_nt(b), full, b->maps_mom, b->cur, b->d_inst,
-                                     d_items, n, mo, b->d_status, b->shared, b->stream);
-        continue;
-      }
+  if constexpr (sizeof(S) == 4) {
+    if (b->vec == 2) {
+      cudaError_t e = cudaSuccess;
+      for (int full = 0; full < 2 && e == cudaSuccess; ++full)
+        if (kind[full])
+          e = lbm::launch_pair_moments(b->rule, mom_nt(b), full, b->maps_mom, b->cur, b->d_inst,
+                                       d_items, n, mo, b->d_status, b->shared, b->stream);
+      return e;
     }
-    e = lbm::launch_sweep<S>(b->rule == lbm::PAIR_PSI64, mom_nt(b), lbm::MODE_MOMENTS, full, (const S*)b->slab[b->cur], nullptr,
-                             b->d_inst, d_items, n, mo, b->d_status, b->stream);
   }
-  return e;
+  const int full = kind[0] && kind[1] ? 2 : kind[1];
+  return lbm::launch_sweep<S>(b->rule == lbm::PAIR_PSI64, mom_nt(b), lbm::MODE_MOMENTS, full,
+                              (const S*)b->slab[b->cur], nullptr, b->d_inst, d_items, n, mo,
+                              b->d_status, b->stream);
 }
 
 // Moments/diagnostics pass over `items` (device list of n entries).

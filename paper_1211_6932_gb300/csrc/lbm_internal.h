@@ -7,9 +7,9 @@
 namespace lbm {
 
 // Launch the fused one-column sweep (MODE_STEP) or its moments/diagnostics pass
-// (MODE_MOMENTS) over n_items work items with nt threads per CTA, in full-width strips or not
-// (see strips_for; a CTA of the moments pass whose instance is of the other kind returns at
-// once); psi64: with the psi_fp64 option (FP32).
+// (MODE_MOMENTS) over n_items work items with nt threads per CTA, in full-width strips (full 1)
+// or not (0; see strips_for), or, the moments pass only, each instance in its own kind (2);
+// psi64: with the psi_fp64 option (FP32).
 template <typename S>
 cudaError_t launch_sweep(bool psi64, int nt, int mode, int full, const S* fin, S* fout, const InstParams* d_inst,
                          const WorkItem* d_items, int n_items, const MomArgs<S>& mo,

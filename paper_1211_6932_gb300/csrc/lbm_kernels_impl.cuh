@@ -40,7 +40,7 @@ static cudaError_t launch_kernel(void (*kernel)(P...), int blocks, int threads, 
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-template <typename S, int NT, int MODE, bool FULL, bool PSI64>
+template <typename S, int NT, int MODE, int FULL, bool PSI64>
 static cudaError_t launch_sweep_cfg(const S* fin, S* fout, const InstParams* d_inst,
                                     const WorkItem* d_items, int n_items, const MomArgs<S>& mo,
                                     int* d_status, cudaStream_t st) {
@@ -60,19 +60,21 @@ static cudaError_t launch_sweep_mode(int mode, int full, const S* fin, S* fout, 
                                      const MomArgs<S>& mo, int* d_status, cudaStream_t st) {
 #define LBM_SWEEP(M, F)                                                                         \
   launch_sweep_cfg<S, NT, M, F, PSI64>(fin, fout, d_inst, d_items, n_items, mo, d_status, st)
-  if (mode == MODE_STEP) return full ? LBM_SWEEP(MODE_STEP, true) : LBM_SWEEP(MODE_STEP, false);
-  return full ? LBM_SWEEP(MODE_MOMENTS, true) : LBM_SWEEP(MODE_MOMENTS, false);
+  if (mode == MODE_STEP) return full ? LBM_SWEEP(MODE_STEP, 1) : LBM_SWEEP(MODE_STEP, 0);
+  return full == 2 ? LBM_SWEEP(MODE_MOMENTS, 2)
+         : full    ? LBM_SWEEP(MODE_MOMENTS, 1)
+                   : LBM_SWEEP(MODE_MOMENTS, 0);
 #undef LBM_SWEEP
 }
 
 template <typename S, int NT>
 static int occupancy_cfg() {
   constexpr size_t smem = SweepCfg<S, NT>::BYTES;
-  cudaFuncSetAttribute(sweep_kernel<S, NT, MODE_STEP, false, false>,
+  cudaFuncSetAttribute(sweep_kernel<S, NT, MODE_STEP, 0, false>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int occ = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &occ, sweep_kernel<S, NT, MODE_STEP, false, false>, NT, smem);
+      &occ, sweep_kernel<S, NT, MODE_STEP, 0, false>, NT, smem);
   return (e == cudaSuccess && occ > 0) ? occ : 1;
 }
 
