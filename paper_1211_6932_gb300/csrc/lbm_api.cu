@@ -1724,6 +1724,10 @@ int diagnostics(Batch* b, lbm_diag* out) {
 // Stop stepping instance i; both slabs then hold its state.
 int freeze(Batch* b, int i) {
   const InstParams& P = b->inst[i];
+  // Full-width strips leave the ghost columns stale, and nothing refreshes those of the other
+  // slab later: a tiling chosen then may sweep the instance in strips, which read them.
+  CK(b, b->fp64 ? lbm::launch_fill_ghosts<double>((double*)b->slab[b->cur], P, b->stream)
+                : lbm::launch_fill_ghosts<float>((float*)b->slab[b->cur], P, b->stream));
   CK(b, cudaMemcpyAsync((char*)b->slab[b->cur ^ 1] + P.off * b->esz,
                         (char*)b->slab[b->cur] + P.off * b->esz, 9 * P.plane * b->esz,
                         cudaMemcpyDeviceToDevice, b->stream));
