@@ -437,6 +437,15 @@ int persist_kind(const Batch* b, int* nt_out = nullptr) {
   return strip && full ? lbm::PERSIST_MIXED : full ? lbm::PERSIST_FULL : lbm::PERSIST_STRIP;
 }
 
+// Rule whose kernels' residency decides between persistent stepping and launches: lattices with
+// the psi_fp64 option, whose kernel has four CTAs an SM instead of five, step persistently from
+// the size on from which those without it do (by their own residency 2317 x 990 would already,
+// and three of them side by side would take 36.1 us a step each instead of 25.6; alone 36.9
+// instead of 41.1).
+int tiling_rule(const Batch* b) {
+  return b->rule == lbm::PAIR_PSI64 ? b->inst[0].visc_mode : b->rule;
+}
+
 // Whether chunks of `rows` rows give the active instances at least two waves of step items
 // (resident persistent CTAs): with fewer, a step's first items would wait on the previous
 // step's last ones, since the odd steps' lists start only half a step further on (the
@@ -451,7 +460,7 @@ bool persist_items_ok(const Batch* b, int rows) {
     if (b->active[i])
       items += (long long)lbm::strips_for(b->inst[i].nx, nt, b->vec) *
                ((b->inst[i].ny + rows - 1) / rows);
-  return items >= 2LL * lbm::persist_occupancy(b->rule, nt, kind) * std::max(b->sms, 1);
+  return items >= 2LL * lbm::persist_occupancy(tiling_rule(b), nt, kind) * std::max(b->sms, 1);
 }
 
 // Whether a batch of both kinds of strips at its default tiling steps with one launch per step
@@ -488,7 +497,7 @@ int default_rows(const Batch* b) {
     if (b->active[i]) {
       const int nt = step_nt(b, i);
       const int occ = b->fp64 ? lbm::sweep_occupancy<double>(nt)
-                      : b->vec == 2 ? lbm::pair_occupancy(b->rule, nt, 8)
+                      : b->vec == 2 ? lbm::pair_occupancy(tiling_rule(b), nt, 8)
                                     : lbm::sweep_occupancy<float>(nt);
       sm_rows += (double)lbm::strips_for(b->inst[i].nx, nt, b->vec) * b->inst[i].ny /
                  std::max(occ, 1);
